@@ -1,11 +1,12 @@
 // X-engine on CUDA cores (Eq. 2, Section 2): the plain baseline and the FP32 path.
 //
-// One CTA computes a 64 x 64 block of input pairs (I-block >= J-block, the lower
-// triangle of Section 4) for one channel; 256 threads each own a 4 x 4 register
-// block of pairs. Spectra are staged in shared memory in chunks, transposed to
-// [spectrum][input] so that every thread reads broadcast / conflict-free.
+// FP32: one CTA per channel and square tile of the lower triangle (Section 4), register
+// tiles (fp32_tile.cuh); one CTA per channel for few inputs.
 //
-//   FP32:  float2 input, V_ij += x_i conj(x_j) with FP32 FFMA.
+// INT8: one CTA computes a 64 x 64 block of input pairs (I-block >= J-block) for one
+// channel; 256 threads each own a 4 x 4 register block of pairs. Spectra are staged in
+// shared memory in chunks, transposed to [spectrum][input] so that every thread reads
+// broadcast / conflict-free.
 //   INT8:  complex int8 input, exact INT32 result with dp4a: a 32-bit word holds
 //          (re, im) of two consecutive spectra, so
 //            Re V_ij += dp4a([re_i im_i ...], [re_j im_j ...])
@@ -13,15 +14,18 @@
 //          with ~re = -re - 1 (bitwise not), representable for every int8 code
 //          including -128 (whose negation is not): the -1 terms sum to -sum(im_j),
 //          which a per-column dp4a with [0 1 0 1] adds back.
+#include <algorithm>
+#include <cmath>
+
+#include "fp32_tile.cuh"
 #include "internal.h"
 
 namespace corr {
 namespace {
 
-constexpr int TB = 64;          // inputs per tile side
-constexpr int NTH = 256;        // threads (16 x 16)
-constexpr int KC_F = 16;        // spectra per chunk, FP32
-constexpr int KC_I = 32;        // spectra per chunk, INT8 (16 words)
+constexpr int TB = 64;          // INT8: inputs per tile side
+constexpr int NTH = 256;        // INT8: threads (16 x 16)
+constexpr int KC_I = 32;        // INT8: spectra per chunk (16 words)
 constexpr int PAD = TB + 1;
 
 __device__ __forceinline__ void tile_of(int t, int &bi, int &bj) {
@@ -33,136 +37,215 @@ __device__ __forceinline__ void tile_of(int t, int &bi, int &bj) {
     bj = t - r * (r + 1) / 2;
 }
 
-__global__ void __launch_bounds__(NTH) k_xeng_f32(const float2 *__restrict__ X, float2 *__restrict__ acc,
-                                                  const float2 *__restrict__ gains, int n_in, int K,
-                                                  long long B, int store) {
-    __shared__ float2 si[KC_F][PAD];
-    __shared__ float2 sj[KC_F][PAD];
+// g_i conj(g_j) v
+__device__ __forceinline__ float2 apply_gains(float2 v, float2 gi, float2 gj) {
+    const float2 w = make_float2(gi.x * gj.x + gi.y * gj.y, gi.y * gj.x - gi.x * gj.y);
+    return make_float2(v.x * w.x - v.y * w.y, v.x * w.y + v.y * w.x);
+}
+
+// FP32 tiles (fp32_tile.cuh): TB = 16 CT inputs square, CT = 2, 3 or 4, one CTA per
+// (channel, lower-triangle tile). On a diagonal tile the warp wholly above the diagonal
+// skips its sums and the rows are loaded once for both sides. Measured against one 64 x 64
+// tile of 4 x 4 sums per 256-thread CTA with synchronous loads: 158 -> 87 us for 130
+// inputs, 64 channels, 500 spectra; 207 -> 60 us for 24 inputs, 256 channels, 1024
+// spectra; 1643 -> 1445 us (47.7 TFLOP/s) for 512 inputs, 64 channels, 1024 spectra.
+template <int CT>
+struct XfCfg {
+    static constexpr int RT = 2 * CT, TB = 16 * CT, P = TB + 2;
+    static constexpr int kSide = kFtKC * P;  // values of one operand of one stage
+    static constexpr size_t smem = sizeof(float2) * 2 * kFtStages * kSide;
+};
+
+template <int CT>
+__global__ void __launch_bounds__(kFtNth, 4) k_xeng_f32(const float2 *__restrict__ X, float2 *__restrict__ acc,
+                                                        const float2 *__restrict__ gains, int n_in, int K,
+                                                        long long B, int n_tiles, int store) {
+    using C = XfCfg<CT>;
+    constexpr int RT = C::RT, TB = C::TB, P = C::P;
+    extern __shared__ __align__(16) float2 sm[];  // [stage][I side, J side][KC][P]
+    const int chan = (int)(blockIdx.x / (unsigned)n_tiles);
     int bi, bj;
-    tile_of(blockIdx.x, bi, bj);
-    const int chan = blockIdx.y;
+    tile_of((int)(blockIdx.x % (unsigned)n_tiles), bi, bj);
+    const bool diag = bi == bj;
     const int I0 = bi * TB, J0 = bj * TB;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
     const float2 *Xc = X + (size_t)chan * n_in * K;
+    const FtPos<RT, CT> pos;
+    const bool live = !(diag && pos.wr < pos.wc);  // this warp's quarter meets the lower triangle
 
-    float ar[4][4], ai[4][4];
+    // loader: spectrum threadIdx.x % 16 of the stage, rows threadIdx.x / 16 + 8 q
+    const int ks = threadIdx.x % kFtKC, row = threadIdx.x / kFtKC;
+    const int n_st = (K + kFtKC - 1) / kFtKC;
+    auto issue = [&](int st) {
+        if (st < n_st) {
+            float2 *sj = sm + ((st % kFtStages) * 2 + 1) * C::kSide + ks * P + row, *si = sj - C::kSide;
+            const int a = st * kFtKC + ks;
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) ar[r][c] = ai[r][c] = 0.0f;
-
-    for (int a0 = 0; a0 < K; a0 += KC_F) {
-#pragma unroll
-        for (int q = 0; q < (TB * KC_F) / NTH; ++q) {
-            int e = threadIdx.x + NTH * q;
-            int row = e / KC_F, a = e % KC_F;
-            int gi = I0 + row, gj = J0 + row, ga = a0 + a;
-            float2 z = make_float2(0.f, 0.f);
-            si[a][row] = (gi < n_in && ga < K) ? __ldg(Xc + (size_t)gi * K + ga) : z;
-            sj[a][row] = (gj < n_in && ga < K) ? __ldg(Xc + (size_t)gj * K + ga) : z;
+            for (int q = 0; q < TB / 8; ++q) {
+                const int gj = J0 + row + 8 * q, gi = I0 + row + 8 * q;
+                const bool lj = gj < n_in && a < K, li = gi < n_in && a < K;
+                ft_copy8(sj + 8 * q, lj ? Xc + (size_t)gj * K + a : X, lj);
+                if (!diag) ft_copy8(si + 8 * q, li ? Xc + (size_t)gi * K + a : X, li);
+            }
         }
-        __syncthreads();
-#pragma unroll 4
-        for (int a = 0; a < KC_F; ++a) {
-            float2 xi[4], xj[4];
+        ft_commit();
+    };
+    float2 sum[RT][CT];
+    ft_zero(sum);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) xi[r] = si[a][ty + 16 * r];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) xj[c] = sj[a][tx + 16 * c];
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    // x_i conj(x_j)
-                    ar[r][c] = fmaf(xi[r].x, xj[c].x, fmaf(xi[r].y, xj[c].y, ar[r][c]));
-                    ai[r][c] = fmaf(xi[r].y, xj[c].x, fmaf(-xi[r].x, xj[c].y, ai[r][c]));
-                }
-        }
-        __syncthreads();
+    for (int st = 0; st < kFtStages - 1; ++st) issue(st);
+    for (int st = 0; st < n_st; ++st) {
+        ft_wait();
+        __syncthreads();  // stage st has landed, and every warp is done with stage st - 1
+        issue(st + kFtStages - 1);
+        const float2 *sj = sm + ((st % kFtStages) * 2 + 1) * C::kSide, *si = diag ? sj : sj - C::kSide;
+        if (live) ft_stage<true, RT, CT, P, P>(sum, si + pos.row0, sj + pos.col0);
     }
+    if (!live) return;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        int i = I0 + ty + 16 * r;
+    for (int r = 0; r < RT; ++r) {
+        const int i = I0 + pos.row(r);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            int j = J0 + tx + 16 * c;
+        for (int c = 0; c < CT; ++c) {
+            const int j = J0 + pos.col(c);
             if (i < n_in && j <= i) {
-                float2 v = make_float2(ar[r][c], ai[r][c]);
-                if (gains) {
-                    float2 gi = __ldg(gains + i), gj = __ldg(gains + j);
-                    // g_i conj(g_j)
-                    float2 w = make_float2(gi.x * gj.x + gi.y * gj.y, gi.y * gj.x - gi.x * gj.y);
-                    v = make_float2(v.x * w.x - v.y * w.y, v.x * w.y + v.y * w.x);
+                float2 v = sum[r][c];
+                if (gains) v = apply_gains(v, __ldg(gains + i), __ldg(gains + j));
+                const size_t b = (size_t)chan * B + (size_t)i * (i + 1) / 2 + j;
+                if (!store) {
+                    const float2 o = acc[b];
+                    v = make_float2(o.x + v.x, o.y + v.y);
                 }
-                size_t b = (size_t)chan * B + (size_t)i * (i + 1) / 2 + j;
-                if (store) {
-                    acc[b] = v;
-                } else {
-                    float2 o = acc[b];
-                    acc[b] = make_float2(o.x + v.x, o.y + v.y);
-                }
+                acc[b] = v;
             }
         }
     }
 }
 
-// Few inputs (n_in <= kSmallIn, at most 253 packed pairs): a 64 x 64 tile would leave
-// most of its threads idle, so one CTA takes one channel and each thread one packed
-// pair (i >= j), the channel's spectra staged in shared memory in chunks of kSmallKC
-// as [spectrum][input]. Four partial sums per pair (spectra a = r mod 4) keep four
-// independent FMA chains in flight; they are added in a fixed order at the end, so
-// the result is run-to-run identical.
-constexpr int kSmallIn = 22;
-constexpr int kSmallKC = 64;
+template <int CT>
+corr_status launch_f32(const Handle &h, const float2 *X, const float2 *gains, bool store, cudaStream_t st) {
+    using C = XfCfg<CT>;
+    const int nb = (h.n_in + C::TB - 1) / C::TB;
+    const long long n_tiles = (long long)nb * (nb + 1) / 2;
+    if (n_tiles * h.n_chan > 0x7fffffffLL) return CORR_EUNSUPPORTED;
+    auto kern = k_xeng_f32<CT>;
+    CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
+    kern<<<(unsigned)(n_tiles * h.n_chan), kFtNth, C::smem, st>>>(X, static_cast<float2 *>(h.acc), gains, h.n_in,
+                                                                 h.n_spectra, h.n_base, (int)n_tiles, store ? 1 : 0);
+    return CORR_OK;
+}
 
-__global__ void __launch_bounds__(NTH) k_xeng_f32_small(const float2 *__restrict__ X, float2 *__restrict__ acc,
-                                                        const float2 *__restrict__ gains, int n_in, int K,
-                                                        long long B, int store) {
-    __shared__ float2 sx[kSmallKC][kSmallIn + 1];
-    const int chan = blockIdx.x;
-    const int p = threadIdx.x;
-    int i = (int)((sqrtf(8.0f * (float)p + 1.0f) - 1.0f) * 0.5f);
-    while ((i + 1) * (i + 2) / 2 <= p) ++i;
-    while (i * (i + 1) / 2 > p) --i;
-    const int j = p - i * (i + 1) / 2;
-    const bool live = p < B;
+// Tile edge of the FP32 X-engine: the one whose busiest SM forms the fewest products,
+// weighed by each tile's rate (operand reads per FMA grow as the tile shrinks). 130 inputs:
+// six tiles of 48 (13,824 products) against six of 64 (24,576) for 8,515 pairs.
+int f32_tile_ct(const Handle &h) {
+    int best = 4;
+    double least = 0.0;
+    for (int ct = 4; ct >= 2; --ct) {
+        const int tb = 16 * ct, nb = (h.n_in + tb - 1) / tb;
+        const double tiles = 0.5 * nb * (nb + 1) - 0.25 * nb;  // diagonal tiles skip a quarter
+        const double per_sm = std::ceil(0.5 * nb * (nb + 1) * h.n_chan / h.n_sm) / (0.5 * nb * (nb + 1));
+        const double cost = tiles * per_sm * tb * tb * (ct == 4 ? 1.0 : ct == 3 ? 1.08 : 1.3);
+        if (ct == 4 || cost < least) best = ct, least = cost;
+    }
+    return best;
+}
+
+// Few inputs (n_in <= kSmallIn): one CTA per channel, one warp per 4 x 4 block of the
+// lower triangle and per K range (n_split of them), one lane per pair of spectra (per
+// spectrum where K is odd), so that the rows are read straight from global memory, 512
+// contiguous bytes per warp and row, and every load feeds four products. The 32 sums of a
+// block (16 pairs, Re and Im) are then added over the lanes by a transposing butterfly
+// that leaves sum number `lane` in each lane, and over the K ranges in order: a fixed
+// order, so the result is run-to-run identical. Bound by the L1 reads (each row is read
+// by the n_in / 4 + 1 blocks it meets) and the FP32 pipe: 14.5 us for 16 inputs, 256
+// channels, 1024 spectra (33.5 MB: 5 us of HBM time), against 30.4 us with one thread per
+// pair reading both factors of each product from shared memory. Above 22 inputs the 32-
+// and 48-input tiles of k_xeng_f32 have the better ratio of sums to reads.
+constexpr int kSmallIn = 22;
+constexpr int kSmallWarps = 21;  // 21 blocks at 22 inputs, else up to 20 warps
+
+template <bool VEC>
+__global__ void __launch_bounds__(32 * kSmallWarps) k_xeng_f32_small(const float2 *__restrict__ X, float2 *__restrict__ acc,
+                                                         const float2 *__restrict__ gains, int n_in, int K,
+                                                         long long B, int n_blk, int n_split, int store) {
+    __shared__ float part[kSmallWarps][32];
+    const int chan = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int blk = warp % n_blk, sp = warp / n_blk;
+    int bi, bj;
+    tile_of(blk, bi, bj);
     const float2 *Xc = X + (size_t)chan * n_in * K;
-    float re[4] = {0.f, 0.f, 0.f, 0.f}, im[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int a0 = 0; a0 < K; a0 += kSmallKC) {
-        for (int e = threadIdx.x; e < n_in * kSmallKC; e += NTH) {
-            const int r = e / kSmallKC, a = e % kSmallKC;
-            sx[a][r] = a0 + a < K ? __ldg(Xc + (size_t)r * K + a0 + a) : make_float2(0.f, 0.f);
-        }
-        __syncthreads();
-        if (live) {
-#pragma unroll 4
-            for (int a = 0; a < kSmallKC; a += 4) {
+    // rows past the end read the last one; their sums are not written
+    const float2 *xi[4], *xj[4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    // x_i conj(x_j)
-                    const float2 xi = sx[a + r][i], xj = sx[a + r][j];
-                    re[r] = fmaf(xi.x, xj.x, fmaf(xi.y, xj.y, re[r]));
-                    im[r] = fmaf(xi.y, xj.x, fmaf(-xi.x, xj.y, im[r]));
-                }
+    for (int r = 0; r < 4; ++r) {
+        xi[r] = Xc + (size_t)min(4 * bi + r, n_in - 1) * K;
+        xj[r] = Xc + (size_t)min(4 * bj + r, n_in - 1) * K;
+    }
+    float v[32];  // sum 2 (4 r + c) + part of pair (4 bi + r, 4 bj + c)
+#pragma unroll
+    for (int e = 0; e < 32; ++e) v[e] = 0.f;
+    auto mac = [&](const float2 (&a)[4], const float2 (&b)[4]) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                // x_i conj(x_j)
+                const int e = 2 * (4 * r + c);
+                v[e] = fmaf(a[r].x, b[c].x, fmaf(a[r].y, b[c].y, v[e]));
+                v[e + 1] = fmaf(a[r].y, b[c].x, fmaf(-a[r].x, b[c].y, v[e + 1]));
             }
+    };
+    const int step = VEC ? 64 : 32;
+    for (int a = sp * step + (VEC ? 2 * lane : lane); a < K; a += n_split * step) {
+        if (VEC) {
+            float2 i0[4], i1[4], j0[4], j1[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(xi[r] + a));
+                i0[r] = make_float2(q.x, q.y), i1[r] = make_float2(q.z, q.w);
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(xj[r] + a));
+                j0[r] = make_float2(q.x, q.y), j1[r] = make_float2(q.z, q.w);
+            }
+            mac(i0, j0);
+            mac(i1, j1);
+        } else {
+            float2 i0[4], j0[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) i0[r] = __ldg(xi[r] + a), j0[r] = __ldg(xj[r] + a);
+            mac(i0, j0);
         }
-        __syncthreads();
     }
-    if (!live) return;
-    float2 v = make_float2((re[0] + re[1]) + (re[2] + re[3]), (im[0] + im[1]) + (im[2] + im[3]));
-    if (gains) {
-        const float2 gi = __ldg(gains + i), gj = __ldg(gains + j);
-        // g_i conj(g_j)
-        const float2 w = make_float2(gi.x * gj.x + gi.y * gj.y, gi.y * gj.x - gi.x * gj.y);
-        v = make_float2(v.x * w.x - v.y * w.y, v.x * w.y + v.y * w.x);
+    // after the step of width o, v[k] holds the sum over the lanes differing in bit o of
+    // sum k (+ o for lanes with that bit set)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            if (k >= o) break;
+            const bool up = (lane & o) != 0;
+            const float send = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
     }
-    const size_t b = (size_t)chan * B + p;
-    if (store) {
-        acc[b] = v;
-    } else {
+    part[warp][lane] = v[0];
+    __syncthreads();
+    if (sp != 0) return;
+    float s = part[warp][lane];
+    for (int q = 1; q < n_split; ++q) s += part[warp + q * n_blk][lane];
+    const float other = __shfl_xor_sync(0xffffffffu, s, 1);
+    const int i = 4 * bi + (lane >> 3), j = 4 * bj + ((lane >> 1) & 3);
+    if ((lane & 1) || i >= n_in || j > i) return;
+    float2 w = make_float2(s, other);
+    if (gains) w = apply_gains(w, __ldg(gains + i), __ldg(gains + j));
+    const size_t b = (size_t)chan * B + (size_t)i * (i + 1) / 2 + j;
+    if (!store) {
         const float2 o = acc[b];
-        acc[b] = make_float2(o.x + v.x, o.y + v.y);
+        w = make_float2(o.x + w.x, o.y + w.y);
     }
+    acc[b] = w;
 }
 
 __device__ __forceinline__ uint32_t rot_word(uint32_t w) {
@@ -266,19 +349,26 @@ __global__ void __launch_bounds__(NTH) k_xeng_i8(const char2 *__restrict__ X, in
 
 corr_status launch_xengine_cudacore(const Handle &h, const void *chan_in, const float2 *gains, bool store,
                                     cudaStream_t st) {
-    const int nb = (h.n_in + TB - 1) / TB;
-    dim3 grid(nb * (nb + 1) / 2, h.n_chan);
     StageScope sc(h, CORR_STAGE_XENGINE, st);
+    corr_status s = CORR_OK;
+    const float2 *X = static_cast<const float2 *>(chan_in);
     if (h.precision == CORR_PREC_INT8) {
+        const int nb = (h.n_in + TB - 1) / TB;
+        dim3 grid(nb * (nb + 1) / 2, h.n_chan);
         k_xeng_i8<<<grid, NTH, 0, st>>>(static_cast<const char2 *>(chan_in), static_cast<int2 *>(h.acc), h.n_in,
                                         h.n_spectra, h.n_base, store ? 1 : 0);
     } else if (h.n_in <= kSmallIn) {
-        k_xeng_f32_small<<<h.n_chan, NTH, 0, st>>>(static_cast<const float2 *>(chan_in),
-                                                   static_cast<float2 *>(h.acc), gains, h.n_in, h.n_spectra,
-                                                   h.n_base, store ? 1 : 0);
+        const int nb = (h.n_in + 3) / 4, n_blk = nb * (nb + 1) / 2;
+        // K ranges: as many warps as fit in 20, as long as each range has a few rounds
+        const int n_split = std::max(1, std::min(20 / n_blk, h.n_spectra / 256));
+        auto kern = (h.n_spectra % 2) == 0 ? k_xeng_f32_small<true> : k_xeng_f32_small<false>;
+        kern<<<h.n_chan, 32 * n_blk * n_split, 0, st>>>(X, static_cast<float2 *>(h.acc), gains, h.n_in, h.n_spectra,
+                                                        h.n_base, n_blk, n_split, store ? 1 : 0);
     } else {
-        k_xeng_f32<<<grid, NTH, 0, st>>>(static_cast<const float2 *>(chan_in), static_cast<float2 *>(h.acc),
-                                         gains, h.n_in, h.n_spectra, h.n_base, store ? 1 : 0);
+        const int ct = f32_tile_ct(h);
+        s = ct == 2 ? launch_f32<2>(h, X, gains, store, st)
+                    : ct == 3 ? launch_f32<3>(h, X, gains, store, st) : launch_f32<4>(h, X, gains, store, st);
+        if (s != CORR_OK) return s;
     }
     return check_launch("k_xeng_cudacore");
 }
