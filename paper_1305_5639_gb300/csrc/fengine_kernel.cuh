@@ -72,7 +72,11 @@ struct FCfg {
     // spectra per CTA: the re-packing modes take 32 up to N = 1024 (64-byte row
     // segments of the planar FP16 planes, 2 CTAs/SM at N = 1024), fewer for longer
     // transforms so that the staging rows stay at 64 KB
-    static constexpr int SB = MODE == kFloatOut ? (N <= 1024 ? 8 : 8192 / N) : (RQ ? (N <= 1024 ? 32 : 32768 / N) : 16);
+    // (the FP32 and power modes take at least the G spectra that are in flight at once: with
+    // 8 spectra per CTA half the threads of N = 256 had no FFT, 15.4 -> 11.5 us for 16
+    // inputs x 1024 spectra)
+    static constexpr int SB = MODE == kFloatOut ? (N <= 1024 ? (G > 8 ? G : 8) : 8192 / N)
+                                                : (RQ ? (N <= 1024 ? 32 : 32768 / N) : (G > 16 ? G : 16));
     // staging row stride in 32-bit words. The re-packing modes stage one 16-bit code
     // pair per (channel k, spectrum s): a row of SB / 2 words whose word index is
     // XOR-swizzled with (k >> SW) & (ROWW - 1), SW = log2(32 / ROWW), so that the
