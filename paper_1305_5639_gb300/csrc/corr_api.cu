@@ -162,10 +162,10 @@ bool use_tc(const Handle &h) {
     return h.precision != CORR_PREC_FP32;  // FP32 has no tensor-core X-engine
 }
 
-// Integration dumps are deferred into the next X-engine launch (whose idle warps run
-// them; see corr_dump) where that launch is long enough to hide them: INT8 and FP16
-// hi/lo on the tensor cores. Plain FP16's X-engine is too short for its FP32 dump
-// (measured: a 2048-input step 37% slower deferred, hi/lo 7% faster, INT8 6% faster).
+// Integration dumps are deferred into the next X-engine launch, whose warps run them
+// beside the MMAs (see corr_dump and SideDump in xengine_tma.cu): INT8 and FP16 hi/lo on
+// the tensor cores. Plain FP16 dumps at once, so that its calls can be captured and
+// replayed as they are issued.
 bool defer_ok(const Handle &h) {
     return (h.precision == CORR_PREC_INT8 || h.precision == CORR_PREC_FP16_HILO) && use_tc(h) &&
            !(h.flags & CORR_FLAG_FUSED_DUMP) && tma_available();

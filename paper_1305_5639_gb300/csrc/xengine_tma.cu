@@ -121,9 +121,8 @@ struct TParams {
     // also written as [block][chan][plane][B] int32 (plane 0 Re, 1 Im), st_nchan channels
     int *st_out;
     int st_kb, st_nchan;
-    // deferred integration dump run by the otherwise idle warps 2 and 3 of every CTA:
-    // side_dst[e] += side_src[e] for e < side_n (int2 for INT8, float2 for FP16), each
-    // CTA a contiguous slice; side_n = 0: none
+    // deferred integration dump (see SideDump): side_dst[e] += side_src[e] for e < side_n
+    // (int2 for INT8, float2 for FP16), each CTA a contiguous slice; side_n = 0: none
     const void *side_src;
     double2 *side_dst;
     long long side_n;
@@ -269,6 +268,69 @@ __device__ __forceinline__ void write_sums16(const int (&R)[64], const Item &itm
     }
 }
 
+// The previous integration's dump into the FP64 long integration, riding along in an
+// X-engine launch. Each CTA owns a contiguous slice, cut into chunks of 256 visibilities
+// that any of its warps claims from a shared counter: warps 2 and 3 (no role in the
+// pipeline) from the start, every other warp once its role has ended. Two warps alone
+// hold too few loads in flight: 38 G visibilities/s, which bound a launch of few spectra
+// (250 inputs, 128 channels, 1504 spectra: 118 -> 91 us with all warps, 76 us without a
+// dump; 128 inputs, 512 channels, 256 spectra: 119 -> 64 us, 37 us without). The
+// sums are exact (integer values below 2^53 for INT8; the FP64 add of the FP32 sums for
+// FP16), as the dump kernel's.
+struct SideState {  // in shared memory, so that the epilogues' registers do not carry it
+    long long lo, hi;         // this CTA's slice
+    unsigned n_chunks, next;  // its chunks, and those claimed so far
+};
+
+template <typename AccT>
+struct SideDump {
+    static constexpr int U = 8;             // visibilities per lane and chunk, loads before stores
+    static constexpr int kChunk = 32 * U;
+    static constexpr unsigned kAhead = 8;   // chunks prefetched into L2 ahead of the claims
+    const TParams &p;
+    volatile SideState *st;  // shared
+    volatile int *abort_flag;
+
+    // bulk L2 prefetch of chunk c of both streams (one lane; 16-byte aligned ranges
+    // inside the buffers)
+    __device__ __forceinline__ void prefetch(unsigned c) const {
+        if (c >= st->n_chunks) return;
+        const long long b = st->lo + (long long)c * kChunk, e = min((long long)st->hi, b + kChunk);
+        const AccT *src = static_cast<const AccT *>(p.side_src);
+        const uintptr_t sa = reinterpret_cast<uintptr_t>(src + b) & ~(uintptr_t)15;
+        const uintptr_t se = reinterpret_cast<uintptr_t>(src + e) & ~(uintptr_t)15;
+        if (se > sa) tc::prefetch_l2_bulk(reinterpret_cast<const void *>(sa), (uint32_t)(se - sa));
+        tc::prefetch_l2_bulk(p.side_dst + b, (uint32_t)((e - b) * sizeof(double2)));
+    }
+    // visibilities 0, 32, 64, ... of a chunk below n (FP64 conversions and adds: beside the
+    // MMAs they cost less than the dump kernel's integer forms, 1740 against 1902 us for
+    // 512 inputs, 512 channels, 4096 spectra)
+    static __device__ __forceinline__ void add(const AccT *s, double2 *d, long long n) {
+        AccT a[U];
+        double2 v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (32 * u < n) {
+                a[u] = __ldcs(s + 32 * u);
+                v[u] = __ldcg(d + 32 * u);
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (32 * u < n) d[32 * u] = make_double2(v[u].x + (double)a[u].x, v[u].y + (double)a[u].y);
+    }
+    // one chunk by the calling warp (all lanes); false when none is left
+    __device__ __forceinline__ bool chunk(int lane) const {
+        unsigned c = 0;
+        if (lane == 0) c = *abort_flag ? st->n_chunks : atomicAdd(const_cast<unsigned *>(&st->next), 1u);
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= st->n_chunks) return false;
+        if (lane == 0) prefetch(c + kAhead);
+        const long long e0 = st->lo + (long long)c * kChunk + lane;
+        add(static_cast<const AccT *>(p.side_src) + e0, p.side_dst + e0, st->hi - e0);
+        return true;
+    }
+};
+
 template <int MODE, class C, bool ST = false, bool WIDE = false>
 __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WIDE : NTHREADS, 1) k_xeng_tma(const __grid_constant__ CUtensorMap tmap,
                                                           const __grid_constant__ CUtensorMap tmapB, const TParams p) {
@@ -298,9 +360,17 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
     const uint32_t drain_bar = bar0 + 8u * (2 * NSTAGE + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sgen + OFF_BAR + 8 * (2 * NSTAGE + 5));
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
+    SideState *side_st = reinterpret_cast<SideState *>(sgen + OFF_BAR + 128);
+    using AccT = typename std::conditional<MODE == kInt8, int2, float2>::type;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
+        if (p.side_n > 0) {
+            side_st->lo = p.side_n * blockIdx.x / gridDim.x;
+            side_st->hi = p.side_n * (blockIdx.x + 1) / gridDim.x;
+            side_st->n_chunks = (unsigned)((side_st->hi - side_st->lo + SideDump<AccT>::kChunk - 1) / SideDump<AccT>::kChunk);
+            side_st->next = 0;
+        }
         for (int s = 0; s < NSTAGE; ++s) {
             tc::mbar_init(full_bar(s), 1);
             tc::mbar_init(empty_bar(s), 1);
@@ -795,51 +865,12 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
         }
     }
 
-    if ((warp == 2 || warp == 3) && p.side_n > 0) {
-        // ------------------------------------------------------------ deferred dump
-        // The previous integration's accumulator into the FP64 long integration, in this
-        // CTA's slice, while the other roles run the X-engine: loads of 8 elements per
-        // thread in flight before their stores. The sums are exact (integer values below
-        // 2^53 for INT8; the FP64 add of the FP32 sums for FP16, as the dump kernel).
-        using AccT = typename std::conditional<MODE == kInt8, int2, float2>::type;
-        const AccT *src = static_cast<const AccT *>(p.side_src);
-        const long long lo = p.side_n * blockIdx.x / gridDim.x, hi = p.side_n * (blockIdx.x + 1) / gridDim.x;
-        constexpr int U = 8;
-        constexpr long long BATCH = 64 * U;  // elements per round of the 64 threads
-        constexpr int AHEAD = 4;              // rounds prefetched into L2 ahead of the loads
-        const int lt = threadIdx.x - 64;  // 0 .. 63
-        // bulk L2 prefetch of rounds [r0, r1) of both streams (one thread; 16-byte aligned
-        // ranges inside the buffers), so that the loads below hit L2
-        auto prefetch = [&](long long e_begin, long long e_end) {
-            e_begin = max(e_begin, lo);
-            e_end = min(e_end, hi);
-            if (e_end <= e_begin) return;
-            const uintptr_t sa = reinterpret_cast<uintptr_t>(src + e_begin) & ~(uintptr_t)15;
-            const uintptr_t se = reinterpret_cast<uintptr_t>(src + e_end) & ~(uintptr_t)15;
-            const uintptr_t da = reinterpret_cast<uintptr_t>(p.side_dst + e_begin);
-            const uintptr_t de = reinterpret_cast<uintptr_t>(p.side_dst + e_end);
-            if (se > sa) tc::prefetch_l2_bulk(reinterpret_cast<const void *>(sa), (uint32_t)(se - sa));
-            tc::prefetch_l2_bulk(reinterpret_cast<const void *>(da), (uint32_t)(de - da));
-        };
-        if (lt == 0) prefetch(lo, lo + AHEAD * BATCH);
-        for (long long e0 = lo + lt; e0 < hi; e0 += BATCH) {
-            if (*abort_flag) break;
-            if (lt == 0) prefetch(e0 + AHEAD * BATCH, e0 + (AHEAD + 1) * BATCH);
-            AccT a[U];
-            double2 v[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long e = e0 + 64 * u;
-                if (e < hi) {
-                    a[u] = __ldcs(src + e);
-                    v[u] = __ldcg(p.side_dst + e);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long e = e0 + 64 * u;
-                if (e < hi) p.side_dst[e] = make_double2(v[u].x + (double)a[u].x, v[u].y + (double)a[u].y);
-            }
+    if (p.side_n > 0) {
+        // deferred dump: warps 2 and 3 from the start, the others when their role has ended
+        const SideDump<AccT> side{p, side_st, abort_flag};
+        if ((warp == 2 || warp == 3) && lane == 0)
+            for (unsigned c = warp - 2; c < SideDump<AccT>::kAhead; c += 2) side.prefetch(c);
+        while (side.chunk(lane)) {
         }
     }
 
@@ -976,7 +1007,7 @@ corr_status launch_xengine_tma_range(const Handle &h, const void *planes, int np
         // the previous integration's deferred dump rides along (all channels, one launch)
         p.side_dst = h.vis64;
         p.side_src = h.pending_src;
-        p.side_n = (long long)h.n_chan * h.n_base;
+        p.side_n = (long long)h.n_chan * h.n_base;  // (small launches: CTAs without tiles join in)
     }
     p.status = h.status;
     p.B = h.n_base;
@@ -992,7 +1023,7 @@ corr_status launch_xengine_tma_range(const Handle &h, const void *planes, int np
         p.st_kb = h.st_block / 64;
         p.st_nchan = h.n_chan;
     }
-    const unsigned grid = (unsigned)(p.n_items < h.n_sm ? p.n_items : h.n_sm);
+    const unsigned grid = (unsigned)(p.n_items < h.n_sm && p.side_n == 0 ? p.n_items : h.n_sm);
     StageScope sc(h, CORR_STAGE_XENGINE, st);
     if (h.precision == CORR_PREC_INT8 && p.st_out) {
         using C = TCfg<2, 64>;
