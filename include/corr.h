@@ -335,7 +335,7 @@ CORR_API corr_status corr_selftest_bounded_wait(int32_t device, int64_t limit_ns
  * counterpart in the paper). */
 enum {
     CORR_STAGE_FENGINE = 0,    /* F-engine FFT + re-packing + corner turn (k_fengine) */
-    CORR_STAGE_PFB = 1,        /* polyphase filter bank FIR pass (k_pfb_fir) */
+    CORR_STAGE_PFB = 1,        /* polyphase filter bank FIR pass (k_pfb_fir), where it is a pass of its own */
     CORR_STAGE_POWER = 2,      /* per-channel power pass */
     CORR_STAGE_PREP = 3,       /* conversion of the X-engine input to planar FP16 operands */
     CORR_STAGE_XENGINE = 4,    /* X-engine (triangle or rectangle) */

@@ -25,7 +25,17 @@ FShape shape_of(const Handle &h) {
     return f;
 }
 
-// With the polyphase filter bank the FIR pass forms the tap-weighted frames of inputs
+// Up to 8 taps on int8 voltages with re-packed output, the filter bank is fused into the
+// F-engine (pfb_frames): the FIR pass wrote 8 bytes per sample and the FFT read them back.
+// 128 inputs x 2 M samples, 4 taps: N = 1024 1361 -> 893 us, N = 256 1101 -> 648, N = 4096
+// 2107 -> 1597; 8 taps at N = 1024 1784 -> 1043. Longer windows (registers per thread), float
+// voltages and the power pass keep the two passes, as does N = 16 (fewer positions than
+// threads).
+bool pfb_fused(const Handle &h) {
+    return h.pfb_win && h.precision == CORR_PREC_INT8 && h.pfb_taps <= 8 && h.n_chan >= 64;
+}
+
+// Otherwise, with the polyphase filter bank the FIR pass forms the tap-weighted frames of inputs
 // [f.i0, f.i0 + n_run) (applying the integer delay advance) into the handle's complex
 // FP32 buffer, and the FFT pass then reads those (float input, phase only).
 corr_status pfb_front(const Handle &h, FShape &f, const void *&volt, cudaStream_t st) {
@@ -69,6 +79,11 @@ corr_status launch_fengine_range(const Handle &h, const void *volt, const float 
     f.i0 = i0;
     f.n_run = n_run;
     if (n_run == 0) return CORR_OK;
+    if (pfb_fused(h)) {
+        StageScope sc(h, CORR_STAGE_FENGINE, st);
+        auto run = h.pfb_taps <= 4 ? fengine_run_pfb4 : fengine_run_pfb8;
+        return run((h.flags & CORR_FLAG_PLANAR) != 0, f, h.pfb_win, h.pfb_taps, volt, scale, out, st);
+    }
     corr_status s = pfb_front(h, f, volt, st);
     if (s != CORR_OK) return s;
     StageScope sc(h, CORR_STAGE_FENGINE, st);

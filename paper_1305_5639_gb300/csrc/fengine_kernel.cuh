@@ -54,7 +54,12 @@ constexpr int kThreads = 256;
 
 enum Mode { kFloatOut = 0, kRequant = 1, kPower = 2, kRequantPlanar = 3 };
 
-template <int N, bool I8, int MODE>
+// Front-end features of one F-engine instantiation: none, delay compensation (an integer
+// advance of the frames and / or the per-channel fractional phase), or the polyphase
+// filter bank formed in shared memory (with or without delays).
+enum Feat { kPlain = 0, kDelay = 1, kPfb = 2 };
+
+template <int N, bool I8, int MODE, int FEAT = kPlain>
 struct FCfg {
     static constexpr int T2 = fengine_t2(N);  // pass-1 threads = pass-2 DFT length
     static constexpr int T1 = N / T2;         // pass-1 DFT length = pass-2 threads
@@ -67,7 +72,10 @@ struct FCfg {
     // 4 EXS / 4 odd per quarter warp, and GS = TG (mod 32) so that the FFTs sharing a
     // warp write to disjoint banks.
     static constexpr int EXS = T2 == 4 ? 8 : T2 + 4;
-    static constexpr int GS = T1 * EXS + (TG >= 32 ? 0 : TG);
+    // The filter bank's frames (complex FP32) are formed in the same per-FFT slots, read
+    // by pass 1 before the exchange overwrites them.
+    static constexpr int GS = (FEAT == kPfb ? 2 * N : T1 * EXS) + (TG >= 32 ? 0 : TG);
+    static_assert(GS >= T1 * EXS, "the exchange fits into a slot");
     static constexpr bool RQ = MODE == kRequant || MODE == kRequantPlanar;
     // spectra per CTA: the re-packing modes take 32 up to N = 1024 (64-byte row
     // segments of the planar FP16 planes, 2 CTAs/SM at N = 1024), fewer for longer
@@ -76,7 +84,8 @@ struct FCfg {
     // 8 spectra per CTA half the threads of N = 256 had no FFT, 15.4 -> 11.5 us for 16
     // inputs x 1024 spectra)
     static constexpr int SB = MODE == kFloatOut ? (N <= 1024 ? (G > 8 ? G : 8) : 8192 / N)
-                                                : (RQ ? (N <= 1024 ? 32 : 32768 / N) : (G > 16 ? G : 16));
+                                                : (RQ ? (FEAT == kPfb && N == 1024 ? 16 : N <= 1024 ? 32 : 32768 / N)
+                                                      : (G > 16 ? G : 16));
     // staging row stride in 32-bit words. The re-packing modes stage one 16-bit code
     // pair per (channel k, spectrum s): a row of SB / 2 words whose word index is
     // XOR-swizzled with (k >> SW) & (ROWW - 1), SW = log2(32 / ROWW), so that the
@@ -137,26 +146,123 @@ __device__ __forceinline__ void cp_async16(void *sdst, const void *gsrc) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// Front-end features of one F-engine instantiation: none, or delay compensation
-// (an integer advance of the frames and / or the per-channel fractional phase).
-enum Feat { kPlain = 0, kDelay = 1 };
+// Polyphase filter-bank parameters of one launch (see pfb_frames).
+struct PfbArgs {
+    const float *win = nullptr;  // [taps][N]
+    int taps = 0;
+};
 
-template <int N, bool I8, int MODE, int FEAT>
+// Where sample n of a filter-bank frame lies in its slot: the 16-byte units of two
+// samples are exchanged in pairs by bit 3 of the unit, so that lanes storing units
+// 2 l, 2 l + 1 of consecutive quads meet every bank once (and pass 1's reads do too).
+__host__ __device__ constexpr int pfb_at(int n) { return n ^ (((n >> 4) & 1) << 1); }
+
+// byte b of u (an offset-binary code x + 128) as the float 12582912 + x + 128
+template <int B>
+__device__ __forceinline__ float ob_float(uint32_t u) {
+    return __uint_as_float(__byte_perm(u, 0x4B400000u, 0x7650 + B));
+}
+
+// The FIR stage of the fused filter bank: frames s0 .. s0 + G - 1 of this CTA into the
+// FFT slots, y_a[n] = sum_{p < taps} h[p][n] s'[(a + p) N + n], taps <= P, int8 voltages.
+// A thread takes four consecutive positions of FR consecutive spectra: each raw quad is
+// loaded (8 bytes) and converted once for all the spectra it enters, the window once.
+// The sums run over p in order with one FMA per tap, as k_pfb_fir's, whose frames these
+// equal bit for bit. At N = 1024 with 4 taps it adds 620 warp instructions per frame to the
+// FFT's 1540 and 96 shared-memory wavefronts to its 290; what bounds the whole is latency:
+// issue 50 % active, the raw loads of a round exposed between two CTA-wide barriers.
+template <int N, int P, int G, int GS>
+__device__ __forceinline__ void pfb_frames(float *slots, const char2 *__restrict__ in, const PfbArgs &f, long long D,
+                                           long long n_rec, int a_first) {
+    // spectra per thread and round (a longer window leaves registers for fewer)
+    constexpr int FR = N >= 1024 ? (P <= 4 ? G : G / 2) : (G * N / 1024 > 0 ? G * N / 1024 : 1);
+    constexpr int NQ = N / 4, UNITS = NQ * (G / FR);
+    static_assert(UNITS % kThreads == 0, "whole rounds");
+    const bool vec = (D & 3) == 0;
+    auto quad = [&](int b, int n) {  // samples n .. n + 3 of frame b of the advanced stream
+        const long long t = (long long)b * N + n + D;
+        uint2 w = make_uint2(0u, 0u);
+        if (t >= n_rec || t + 4 <= 0) return w;
+        if (vec) {  // n_rec and t are multiples of 4: wholly inside
+            w = __ldg(reinterpret_cast<const uint2 *>(in + t));
+        } else {
+            const unsigned short *s = reinterpret_cast<const unsigned short *>(in) + t;
+            uint32_t e[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) e[x] = t + x >= 0 && t + x < n_rec ? (uint32_t)__ldg(s + x) : 0u;
+            w = make_uint2(e[0] | (e[1] << 16), e[2] | (e[3] << 16));
+        }
+        return w;
+    };
+#pragma unroll 1
+    for (int u = threadIdx.x; u < UNITS; u += kThreads) {
+        const int n = 4 * (u % NQ), g0 = (u / NQ) * FR, a0 = a_first + g0;
+        // every load of the round in flight together
+        float4 h[P];
+#pragma unroll
+        for (int p = 0; p < P; ++p)
+            h[p] = p < f.taps ? __ldg(reinterpret_cast<const float4 *>(f.win + (size_t)p * N + n)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        uint2 raw[FR + P - 1];
+        const long long t0 = (long long)a0 * N + n + D;
+        if (vec && t0 >= 0 && t0 + (long long)(FR + P - 2) * N < n_rec) {
+            const char2 *src = in + t0;
+#pragma unroll
+            for (int q = 0; q < FR + P - 1; ++q) raw[q] = __ldg(reinterpret_cast<const uint2 *>(src + q * N));
+        } else {
+#pragma unroll
+            for (int q = 0; q < FR + P - 1; ++q) raw[q] = quad(a0 + q, n);
+        }
+        float2 y[FR][4];
+#pragma unroll
+        for (int r = 0; r < FR; ++r)
+#pragma unroll
+            for (int x = 0; x < 4; ++x) y[r][x] = make_float2(0.f, 0.f);
+        // raw quad q enters spectra r = q - p: converted once, p ascending for every r
+#pragma unroll
+        for (int q = 0; q < FR + P - 1; ++q) {
+            const uint32_t a = raw[q].x ^ 0x80808080u, b = raw[q].y ^ 0x80808080u;
+            const float2 off = make_float2(kMagic + 128.0f, kMagic + 128.0f);
+            const float2 x0 = f2_sub(make_float2(ob_float<0>(a), ob_float<1>(a)), off);
+            const float2 x1 = f2_sub(make_float2(ob_float<2>(a), ob_float<3>(a)), off);
+            const float2 x2 = f2_sub(make_float2(ob_float<0>(b), ob_float<1>(b)), off);
+            const float2 x3 = f2_sub(make_float2(ob_float<2>(b), ob_float<3>(b)), off);
+#pragma unroll
+            for (int p = 0; p < P; ++p) {
+                const int r = q - p;
+                if (r < 0 || r >= FR) continue;
+                y[r][0] = f2_fma(make_float2(h[p].x, h[p].x), x0, y[r][0]);
+                y[r][1] = f2_fma(make_float2(h[p].y, h[p].y), x1, y[r][1]);
+                y[r][2] = f2_fma(make_float2(h[p].z, h[p].z), x2, y[r][2]);
+                y[r][3] = f2_fma(make_float2(h[p].w, h[p].w), x3, y[r][3]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < FR; ++r) {
+            float2 *slot = reinterpret_cast<float2 *>(slots + (size_t)(g0 + r) * GS);
+            *reinterpret_cast<float4 *>(slot + pfb_at(n)) = make_float4(y[r][0].x, y[r][0].y, y[r][1].x, y[r][1].y);
+            *reinterpret_cast<float4 *>(slot + pfb_at(n + 2)) = make_float4(y[r][2].x, y[r][2].y, y[r][3].x, y[r][3].y);
+        }
+    }
+}
+
+template <int N, bool I8, int MODE, int FEAT, int P = 0>
 __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >= 512)) ? 1 : (N >= 512 ? 2 : 3)) k_fengine(const void *__restrict__ volt,
                                                       const float *__restrict__ scale,
                                                       void *__restrict__ out,
                                                       double *__restrict__ power, int n_in, int K,
                                                       const float2 *__restrict__ tw_glob, int i0, int vec_out,
                                                       const int *__restrict__ dint,
-                                                      const float2 *__restrict__ dph, int async_raw) {
-    using C = FCfg<N, I8, MODE>;
+                                                      const float2 *__restrict__ dph, int async_raw,
+                                                      const PfbArgs pfb) {
+    using C = FCfg<N, I8, MODE, FEAT>;
     constexpr int T1 = C::T1, T2 = C::T2, TG = C::TG, G = C::G, EXS = C::EXS, SB = C::SB, ROWW = C::ROWW;
     constexpr int TV = T1 > T2 ? T1 : T2;  // register values per thread
     // square 32- or 64-point passes read the exchange into float arrays and do pass 2's
     // first stage in scalar arithmetic (no register moves into the (re, im) pairs); the
     // smaller lengths keep the in-place reads, which fit their register budgets
     constexpr bool kScalarStage = T1 == T2 && T2 >= 32;
-    constexpr bool DLY = FEAT == kDelay;  // delay code compiled in
+    constexpr bool PFB = FEAT == kPfb;
+    constexpr bool DLY = FEAT != kPlain;  // delay code compiled in
     // int8 samples enter the plain FFT scaled by 256 on an offset (i8_to_f2_scaled); the
     // delay instantiation converts them exactly (measured faster there)
     constexpr bool SCALED = I8 && !DLY;
@@ -221,7 +327,12 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
     }
     // per-CTA copy of the twiddle table (shared-memory loads in the FFT loop; measured
     // faster than L1 lookups, while the channel scales are faster from L1)
-    for (int m = threadIdx.x; m < N; m += kThreads) {
+    const bool tw_async = PFB && !has_dly;  // as it stands: in flight while the first frames form
+    if (tw_async) {
+        for (int m = 2 * threadIdx.x; m < N; m += 2 * kThreads) cp_async16(tws + m, tw_glob + m);
+        cp_async_commit();
+    }
+    for (int m = threadIdx.x; m < N && !tw_async; m += kThreads) {
         float2 w = __ldg(tw_glob + m);
         if (DLY && has_dly) {
             w = cmul(w, __ldg(dph + (size_t)i * (T1 + T2) + m / T2));  // table [k1][t]: c[k1]
@@ -231,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
         tws[m] = w;
         if constexpr (MODE == kPower) scs[m] = 0.0f;
     }
-    __syncthreads();
+    if constexpr (!PFB) __syncthreads();
 
     const int g = threadIdx.x / TG;
     const int t = threadIdx.x % TG;
@@ -257,7 +368,17 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
         const long long base = (long long)i * n_rec + off + t;
         // with delays, frames that reach outside the record take the checked loads
         const bool inside = !DLY || (off >= 0 && off + N <= n_rec);
-        if constexpr (I8) {
+        if constexpr (PFB) {
+            if (s0 > 0) __syncthreads();  // every FFT has left its slot
+            pfb_frames<N, P, G, C::GS>(ex, reinterpret_cast<const char2 *>(volt) + (size_t)i * n_rec, pfb, D, n_rec,
+                                       a0 + s0);
+            cp_async_wait_all();
+            __syncthreads();
+            const float2 *frame = reinterpret_cast<const float2 *>(exg);
+#pragma unroll
+            for (int m = 0; m < T1; ++m) v[m] = valid1 ? frame[pfb_at(t + T2 * m)] : make_float2(0.f, 0.f);
+            group_sync();  // read before the exchange overwrites the slot
+        } else if constexpr (I8) {
             const unsigned short *src = reinterpret_cast<const unsigned short *>(volt) + base;
             if (use_async) {
                 cp_async_wait_all();
@@ -374,12 +495,20 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
             if (use_async && s0 + G < SB) issue_raw(s0 + G + g);  // next frame into the free buffer
             fft_dif<T2>(v);  // v[bitrev(k2)] = X[t + T1 k2]
         }
+        if (PFB && has_dly) {
+            // delay phases exp(+j 2 pi T1 k2 f / N), in a block of their own: without delays
+            // the plain filter bank skips it as a whole
+            sfor<1, T2>([&](auto K2) {
+                constexpr int k2 = decltype(K2)::value;
+                v[bitrev(k2, ilog2(T2))] = cmul(v[bitrev(k2, ilog2(T2))], dsm[k2]);
+            });
+        }
         if (valid && act2) {
             sfor<0, T2>([&](auto K2) {
                 constexpr int k2 = decltype(K2)::value;
                 const int k = t + T1 * k2;
                 float2 x = v[bitrev(k2, ilog2(T2))];
-                if constexpr (DLY && k2 != 0) {
+                if constexpr (FEAT == kDelay && k2 != 0) {
                     if (has_dly) x = cmul(x, dsm[k2]);  // delay phase exp(+j 2 pi T1 k2 f / N)
                 }
                 if constexpr (MODE == kRequant || MODE == kRequantPlanar) {
@@ -470,11 +599,11 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
     }
 }
 
-template <int N, bool I8, int MODE, int FEAT>
+template <int N, bool I8, int MODE, int FEAT, int P = 0>
 corr_status launch_one_(const FShape &f, const void *volt, const float *scale, void *out, double *power,
-                       cudaStream_t st) {
-    using C = FCfg<N, I8, MODE>;
-    auto kern = k_fengine<N, I8, MODE, FEAT>;
+                       cudaStream_t st, const PfbArgs &pfb = {}) {
+    using C = FCfg<N, I8, MODE, FEAT>;
+    auto kern = k_fengine<N, I8, MODE, FEAT, P>;
     CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
     // 16-byte row stores need 16-byte aligned rows: an aligned buffer and 8 | n_spectra
     const int vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0) && (f.n_spectra % 8 == 0);
@@ -485,7 +614,7 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     // public entry points only accept 16-byte aligned voltages, so this is a safeguard
     const int async_raw = reinterpret_cast<uintptr_t>(volt) % 16 == 0;
     kern<<<grid, kThreads, C::smem, st>>>(volt, scale, out, power, f.n_in, f.n_spectra, f.tw, f.i0, vec_out,
-                                          f.dint, f.dph, async_raw);
+                                          f.dint, f.dph, async_raw, pfb);
     return check_launch("k_fengine");
 }
 
@@ -498,6 +627,27 @@ corr_status launch_mode(const FShape &f, const void *volt, const float *scale, v
                     : launch_one_<NN, false, MODE, FEAT>(f, volt, scale, out, power, st);
     switch (f.n_chan) {
         CORR_F_CASE(16)
+        CORR_F_CASE(64)
+        CORR_F_CASE(128)
+        CORR_F_CASE(256)
+        CORR_F_CASE(512)
+        CORR_F_CASE(1024)
+        CORR_F_CASE(2048)
+        CORR_F_CASE(4096)
+        default: return CORR_EUNSUPPORTED;
+    }
+#undef CORR_F_CASE
+}
+
+// The fused filter bank of up to P taps: int8 voltages, re-packed output.
+template <int P>
+corr_status launch_pfb(bool planar, const FShape &f, const PfbArgs &pfb, const void *volt, const float *scale, void *out,
+                       cudaStream_t st) {
+#define CORR_F_CASE(NN)                                                                                           \
+    case NN:                                                                                                      \
+        return planar ? launch_one_<NN, true, kRequantPlanar, kPfb, P>(f, volt, scale, out, nullptr, st, pfb)     \
+                      : launch_one_<NN, true, kRequant, kPfb, P>(f, volt, scale, out, nullptr, st, pfb);
+    switch (f.n_chan) {
         CORR_F_CASE(64)
         CORR_F_CASE(128)
         CORR_F_CASE(256)
@@ -530,5 +680,10 @@ corr_status fengine_run_plain(int mode, const FShape &f, const void *volt, const
                               double *power, cudaStream_t st);
 corr_status fengine_run_delay(int mode, const FShape &f, const void *volt, const float *scale, void *out,
                               double *power, cudaStream_t st);
+// Fused filter bank, win [taps][n_chan]: taps <= 4 and <= 8.
+corr_status fengine_run_pfb4(bool planar, const FShape &f, const float *win, int taps, const void *volt,
+                             const float *scale, void *out, cudaStream_t st);
+corr_status fengine_run_pfb8(bool planar, const FShape &f, const float *win, int taps, const void *volt,
+                             const float *scale, void *out, cudaStream_t st);
 
 }  // namespace corr

@@ -1,4 +1,5 @@
-// Polyphase filter-bank front end: the FIR pass. For spectrum a of input i it forms
+// Polyphase filter-bank front end: the FIR pass, where the filter bank is not fused into
+// the F-engine (see pfb_fused in fengine.cu). For spectrum a of input i it forms
 //     y_a[n] = sum_{p < P} h[p][n] s'_i[(a + p) N + n],    n < N,
 // with s'_i[t] = s_i[t + D_i] (the integer delay advance, D_i = 0 without delays)
 // and zero wherever t + D_i is not a recorded sample, and writes the frames as
