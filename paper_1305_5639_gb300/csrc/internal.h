@@ -43,6 +43,9 @@ struct Handle {
     const void *pending_src = nullptr;
     int64_t acc_spectra = 0;     // spectra accumulated since the last dump (INT8 overflow guard)
     double2 *vis64 = nullptr;    // FP64 long-integration buffer [n_chan][B]
+    bool vis_zero = false;       // vis64 known to be all-zero (zeroed by a reset, nothing added since)
+    bool captured = false;       // a call on this handle was stream-captured: its replays may change
+                                 // the buffers without the flags above knowing
     float2 *twiddle = nullptr;   // F-engine twiddles W_N^(t k1), [k1][t], N = T1 x T2
     void *ftc_b = nullptr;       // tensor-core F-engine DFT matrices F_h, F_l (N = 1024, INT8)
     int32_t *dly_int = nullptr;  // delay compensation (null: off): integer advance per input
