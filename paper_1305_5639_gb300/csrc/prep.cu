@@ -191,32 +191,39 @@ void launch_np(bool vec, unsigned blocks, const float2 *X, uint2 *out, float *rs
 // integers, exact in FP16), zeros past K: one thread per 8 spectra of one row.
 // x ^ 0x80 is the offset-binary code x + 128; under the high byte 0x64 it is the
 // FP16 value 1024 + (x + 128), from which 1152 is subtracted exactly.
-template <bool VEC>
-__global__ void __launch_bounds__(256) k_i8_to_planar(const char2 *__restrict__ X, uint4 *__restrict__ out,
-                                                      long long n_chunks, int n_in, int K, int Kp) {
-    const int cpr = Kp / 8;  // 8-spectrum chunks per padded row
+// VB: bytes per load, the largest of 16, 8, 4, 2 that divides a row's bytes (2 K), so that
+// every chunk starts on that boundary; I: index type (32 bits where all chunks fit: the
+// two divisions per chunk are most of its integer work).
+template <int VB, typename I>
+__global__ void __launch_bounds__(256) k_i8_to_planar(const char2 *__restrict__ X, uint4 *__restrict__ out, I n_chunks,
+                                                      int n_in, int K, int Kp) {
+    const I cpr = (I)(Kp / 8);  // 8-spectrum chunks per padded row
     const uint32_t k1152 = 0x64806480u;
-    for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n_chunks;
-         q += (long long)gridDim.x * blockDim.x) {
-        const long long row = q / cpr;
+    for (I q = (I)blockIdx.x * blockDim.x + threadIdx.x; q < n_chunks; q += (I)gridDim.x * blockDim.x) {
+        const I row = q / cpr;
         const int s0 = 8 * (int)(q - row * cpr);
-        const char2 *x = X + row * K;
-        uint32_t w[4];
-        if (VEC) {  // K % 8 == 0: rows and chunks are 16-byte aligned
-            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x + s0));
+        const char2 *x = X + (long long)row * K + s0;
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        if constexpr (VB == 16) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(x));
             w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
+        } else if constexpr (VB == 8) {  // K a multiple of 4: each half chunk wholly in or out
+            const uint2 lo = __ldg(reinterpret_cast<const uint2 *>(x));
+            w[0] = lo.x, w[1] = lo.y;
+            if (s0 + 4 < K) {
+                const uint2 hi = __ldg(reinterpret_cast<const uint2 *>(x) + 1);
+                w[2] = hi.x, w[3] = hi.y;
+            }
+        } else if constexpr (VB == 4) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (s0 + 2 * e < K) w[e] = __ldg(reinterpret_cast<const unsigned int *>(x) + e);
         } else {
+            const unsigned short *u = reinterpret_cast<const unsigned short *>(x);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                uint32_t lo = 0, hi = 0;
-                if (s0 + 2 * e < K) {
-                    const char2 c = x[s0 + 2 * e];
-                    lo = (uint32_t)(uint8_t)c.x | ((uint32_t)(uint8_t)c.y << 8);
-                }
-                if (s0 + 2 * e + 1 < K) {
-                    const char2 c = x[s0 + 2 * e + 1];
-                    hi = (uint32_t)(uint8_t)c.x | ((uint32_t)(uint8_t)c.y << 8);
-                }
+                const uint32_t lo = s0 + 2 * e < K ? (uint32_t)__ldg(u + 2 * e) : 0u;
+                const uint32_t hi = s0 + 2 * e + 1 < K ? (uint32_t)__ldg(u + 2 * e + 1) : 0u;
                 w[e] = lo | (hi << 16);
             }
         }
@@ -234,12 +241,22 @@ __global__ void __launch_bounds__(256) k_i8_to_planar(const char2 *__restrict__ 
             im[e] = h2u(hi);
         }
         // zero codes past K (the offset arithmetic above maps a zero byte pair to 0 already)
-        const long long chan = row / n_in;
-        const int in = (int)(row - chan * n_in);
-        const long long o = ((chan * 2) * n_in + in) * (long long)cpr + s0 / 8;
+        const I chan = row / (I)n_in;
+        const int in = (int)(row - chan * (I)n_in);
+        const long long o = ((long long)chan * 2 * n_in + in) * (long long)cpr + s0 / 8;
         out[o] = make_uint4(re[0], re[1], re[2], re[3]);
         out[o + (long long)n_in * cpr] = make_uint4(im[0], im[1], im[2], im[3]);
     }
+}
+
+template <int VB>
+void launch_i8(unsigned blocks, const void *X, void *ws, long long n_chunks, int n_in, int K, int Kp, cudaStream_t st) {
+    const char2 *x = static_cast<const char2 *>(X);
+    uint4 *o = static_cast<uint4 *>(ws);
+    if (n_chunks < (1ll << 31))
+        k_i8_to_planar<VB, unsigned><<<blocks, 256, 0, st>>>(x, o, (unsigned)n_chunks, n_in, K, Kp);
+    else
+        k_i8_to_planar<VB, long long><<<blocks, 256, 0, st>>>(x, o, n_chunks, n_in, K, Kp);
 }
 
 }  // namespace
@@ -252,13 +269,14 @@ corr_status launch_i8_to_planar(const Handle &h, const void *X, void *ws, cudaSt
     long long blocks = (n_chunks + 255) / 256;
     const long long cap = (long long)h.n_sm * 16;
     if (blocks > cap) blocks = cap;
-    const bool vec = (K % 8) == 0 && (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
-    if (vec)
-        k_i8_to_planar<true><<<(unsigned)blocks, 256, 0, st>>>(static_cast<const char2 *>(X), static_cast<uint4 *>(ws),
-                                                               n_chunks, h.n_in, K, Kp);
-    else
-        k_i8_to_planar<false><<<(unsigned)blocks, 256, 0, st>>>(static_cast<const char2 *>(X),
-                                                                static_cast<uint4 *>(ws), n_chunks, h.n_in, K, Kp);
+    // (the public entry points take 16-byte aligned data only; 250 inputs x 128 channels x
+    // 1500 spectra, K a multiple of 4: 55 -> 47.5 us against single samples)
+    const bool al = (reinterpret_cast<uintptr_t>(X) & 15u) == 0;
+    const unsigned nb = (unsigned)blocks;
+    if (al && (K % 8) == 0) launch_i8<16>(nb, X, ws, n_chunks, h.n_in, K, Kp, st);
+    else if (al && (K % 4) == 0) launch_i8<8>(nb, X, ws, n_chunks, h.n_in, K, Kp, st);
+    else if (al && (K % 2) == 0) launch_i8<4>(nb, X, ws, n_chunks, h.n_in, K, Kp, st);
+    else launch_i8<2>(nb, X, ws, n_chunks, h.n_in, K, Kp, st);
     return check_launch("k_i8_to_planar");
 }
 
