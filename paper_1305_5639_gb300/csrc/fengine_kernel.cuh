@@ -529,7 +529,6 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
         const int nv = min(SB, K - a0);
         if constexpr (MODE == kRequantPlanar || MODE == kRequant) {
             uint16_t *dst = reinterpret_cast<uint16_t *>(out);
-            const uint16_t *sh = reinterpret_cast<const uint16_t *>(stg);
             // planar FP16 layout [k][plane][i][a]; int8 layout [k][i][a] (complex int8)
             constexpr int PL = MODE == kRequantPlanar ? 2 : 1;
             if (nv == SB && vec_out) {
@@ -562,18 +561,27 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
                     }
                 }
             } else {
-                for (int e = threadIdx.x; e < N * SB; e += kThreads) {
-                    const int k = e / SB, c = e % SB;
-                    if (c < nv) {
-                        const uint16_t code = sh[slot(k, c)];
-                        uint16_t *row0 = dst + ((size_t)(PL * k) * n_in + i) * K + a0;
+                // unaligned rows or a short last block: a thread per code, whole rows per store
+                // instruction (one write request per row), U staged codes in flight
+                constexpr int U = 8, RPI = kThreads / SB;  // rows per round
+                const uint16_t *sh = reinterpret_cast<const uint16_t *>(stg);
+                const size_t plane = (size_t)n_in * K;
+                const int c = threadIdx.x % SB;
+                for (int k0 = threadIdx.x / SB; c < nv && k0 < N; k0 += U * RPI) {
+                    uint32_t code[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) code[u] = k0 + u * RPI < N ? sh[slot(k0 + u * RPI, c)] : 0u;
+                    uint16_t *d = dst + ((size_t)(PL * k0) * n_in + i) * K + a0 + c;
+#pragma unroll
+                    for (int u = 0; u < U; ++u, d += PL * RPI * plane) {
+                        if (k0 + u * RPI >= N) break;
                         if constexpr (MODE == kRequantPlanar) {
                             uint32_t re, im;
-                            ob_codes_to_f16_planes((uint32_t)code, re, im);
-                            row0[c] = (uint16_t)(re & 0xffffu);
-                            row0[(size_t)n_in * K + c] = (uint16_t)(im & 0xffffu);
+                            ob_codes_to_f16_planes(code[u], re, im);
+                            d[0] = (uint16_t)re;
+                            d[plane] = (uint16_t)im;
                         } else {
-                            row0[c] = code;
+                            d[0] = (uint16_t)code[u];
                         }
                     }
                 }
