@@ -10,9 +10,10 @@
 //   exchange through shared memory (padded rows, conflict-free)
 //   pass 2: thread k1 < T1 holds Y[t][k1], t < T2, and computes the T2-point DFT
 //           over t, giving X[k1 + T1 k2].
-// Square lengths (16, 64, 256, 1024) keep every thread busy in both passes; the
-// others (128, 512, 2048, 4096: T2 = 2 T1 or T1 = T2 = 64) leave the threads past
-// the shorter dimension idle in one pass.
+// Square lengths (16, 64, 256, 1024) take one thread per column and per row. For T2 = 2 T1
+// (128, 512, 2048) two threads share each row's T2-point DFT, and for 64 x 64 (4096) each
+// column's and each row's (dft_shared): every thread is busy in both passes and holds at
+// most 32 values, so that 16 warps fit on an SM.
 // A CTA handles one input and SB consecutive spectra; the outputs are staged in
 // shared memory as [channel][spectrum] so that every (channel, input) row segment
 // of SB spectra is written to global memory contiguously (the corner turn). Raw
@@ -50,8 +51,6 @@ struct FShape {
 namespace {
 
 
-constexpr int kThreads = 256;
-
 enum Mode { kFloatOut = 0, kRequant = 1, kPower = 2, kRequantPlanar = 3 };
 
 // Front-end features of one F-engine instantiation: none, delay compensation (an integer
@@ -64,8 +63,18 @@ struct FCfg {
     static constexpr int T2 = fengine_t2(N);  // pass-1 threads = pass-2 DFT length
     static constexpr int T1 = N / T2;         // pass-1 DFT length = pass-2 threads
     static_assert(T2 > 0 && T1 * T2 == N && T1 <= T2 && T2 <= 64, "unsupported F-engine length");
-    static constexpr int TG = T2;             // threads per FFT group
-    static constexpr int G = kThreads / TG;   // FFTs in flight per CTA
+    static constexpr int H1 = T1 == 64 ? 2 : 1;             // threads per column in pass 1
+    static constexpr int H2 = T2 == 2 * T1 || T1 == 64 ? 2 : 1;  // threads per row in pass 2
+    static constexpr int TG = T2 * H1;        // threads per FFT group
+    static_assert(TG == T1 * H2, "every thread takes part in both passes");
+    static constexpr bool RQ = MODE == kRequant || MODE == kRequantPlanar;
+    // long re-packed transforms read the twiddles through L1 instead of a shared-memory copy,
+    // so that two CTAs fit on an SM at N = 2048 (one's copy-out beside the other's FFTs: 370
+    // -> 324 us below) and twice the staging rows at N = 4096
+    static constexpr bool TWG = N >= 2048 && RQ && FEAT != kPfb;
+    // threads per CTA: 256, or 512 where the shared memory leaves room for one CTA only
+    static constexpr int NT = (N >= 2048 && RQ && !TWG) || (N == 4096 && RQ) ? 512 : 256;
+    static constexpr int G = NT / TG;         // FFTs in flight per CTA
     // Exchange buffer of one FFT: T1 rows of EXS floats; row k1 receives Y[0..T2-1][k1]
     // (one column per writing thread) and is read back as float4. EXS and the per-FFT
     // stride GS keep both the scalar writes and the float4 reads free of bank conflicts:
@@ -76,15 +85,16 @@ struct FCfg {
     // by pass 1 before the exchange overwrites them.
     static constexpr int GS = (FEAT == kPfb ? 2 * N : T1 * EXS) + (TG >= 32 ? 0 : TG);
     static_assert(GS >= T1 * EXS, "the exchange fits into a slot");
-    static constexpr bool RQ = MODE == kRequant || MODE == kRequantPlanar;
     // spectra per CTA: the re-packing modes take 32 up to N = 1024 (64-byte row
-    // segments of the planar FP16 planes, 2 CTAs/SM at N = 1024), fewer for longer
-    // transforms so that the staging rows stay at 64 KB
+    // segments of the planar FP16 planes, 2 CTAs/SM at N = 1024), 16 for longer
+    // transforms: whole 32-byte sectors per row (with 8 at N = 4096, whose staging rows
+    // then leave room for two CTAs, the planar layout took 674 us against 489 for 64
+    // inputs x 512 spectra)
     // (the FP32 and power modes take at least the G spectra that are in flight at once: with
     // 8 spectra per CTA half the threads of N = 256 had no FFT, 15.4 -> 11.5 us for 16
     // inputs x 1024 spectra)
     static constexpr int SB = MODE == kFloatOut ? (N <= 1024 ? (G > 8 ? G : 8) : 8192 / N)
-                                                : (RQ ? (FEAT == kPfb && N == 1024 ? 16 : N <= 1024 ? 32 : 32768 / N)
+                                                : (RQ ? (FEAT == kPfb && N == 1024 ? 16 : N <= 1024 ? 32 : (N == 4096 && FEAT != kPfb) ? 16 : 32768 / N)
                                                       : (G > 16 ? G : 16));
     // staging row stride in 32-bit words. The re-packing modes stage one 16-bit code
     // pair per (channel k, spectrum s): a row of SB / 2 words whose word index is
@@ -97,7 +107,7 @@ struct FCfg {
     static_assert(!RQ || (ROWW >= 4 && ROWW <= 16), "swizzle assumes 4..16-word rows");
     static constexpr size_t ex_bytes = sizeof(float) * (size_t)G * GS;
     static constexpr size_t pw_bytes = MODE == kPower ? sizeof(float) * N : 0;
-    static constexpr size_t tw_bytes = sizeof(float2) * (size_t)N;  // twiddle table copy
+    static constexpr size_t tw_bytes = TWG ? 0 : sizeof(float2) * (size_t)N;  // twiddle table copy
     static constexpr size_t dl_bytes = sizeof(float2) * 64;         // delay phases d[k2] (T2 <= 64)
     static constexpr size_t st_bytes = sizeof(uint32_t) * (size_t)N * ROWW;
     static constexpr size_t smem = ex_bytes + pw_bytes + tw_bytes + dl_bytes + st_bytes;
@@ -171,13 +181,13 @@ __device__ __forceinline__ float ob_float(uint32_t u) {
 // equal bit for bit. At N = 1024 with 4 taps it adds 620 warp instructions per frame to the
 // FFT's 1540 and 96 shared-memory wavefronts to its 290; what bounds the whole is latency:
 // issue 50 % active, the raw loads of a round exposed between two CTA-wide barriers.
-template <int N, int P, int G, int GS>
+template <int N, int P, int G, int GS, int NT>
 __device__ __forceinline__ void pfb_frames(float *slots, const char2 *__restrict__ in, const PfbArgs &f, long long D,
                                            long long n_rec, int a_first) {
     // spectra per thread and round (a longer window leaves registers for fewer)
     constexpr int FR = N >= 1024 ? (P <= 4 ? G : G / 2) : (G * N / 1024 > 0 ? G * N / 1024 : 1);
     constexpr int NQ = N / 4, UNITS = NQ * (G / FR);
-    static_assert(UNITS % kThreads == 0, "whole rounds");
+    static_assert(UNITS % NT == 0, "whole rounds");
     const bool vec = (D & 3) == 0;
     auto quad = [&](int b, int n) {  // samples n .. n + 3 of frame b of the advanced stream
         const long long t = (long long)b * N + n + D;
@@ -195,7 +205,7 @@ __device__ __forceinline__ void pfb_frames(float *slots, const char2 *__restrict
         return w;
     };
 #pragma unroll 1
-    for (int u = threadIdx.x; u < UNITS; u += kThreads) {
+    for (int u = threadIdx.x; u < UNITS; u += NT) {
         const int n = 4 * (u % NQ), g0 = (u / NQ) * FR, a0 = a_first + g0;
         // every load of the round in flight together
         float4 h[P];
@@ -245,8 +255,45 @@ __device__ __forceinline__ void pfb_frames(float *slots, const char2 *__restrict
     }
 }
 
+// One L-point DFT shared by two threads of a warp, the lanes of which differ in bit HB:
+// thread h holds x[q h + i] (lo[i]) and x[L/2 + q h + i] (hi[i]), i < q = L/4, and returns in
+// v[bitrev(k')] the outputs k = 2 k' + h. The first radix-2 stage pairs what a thread holds;
+// thread 0 then goes on with the sums and thread 1 with the differences, of which each gets
+// the other half from its partner (in the second stage the two halves meet: the thread that
+// holds the upper ones subtracts the wrong way round, put right by an exact factor -1). The
+// butterflies, factors and roundings are fft_dif<L>'s: the results are the same. 64 inputs,
+// int8 layout (us): N = 2048 x 1024 spectra 555 -> 324 (the T2-point DFTs ran on one of two
+// warps, at 212 registers and 8 warps per SM), N = 4096 x 512 527 -> 445 (8 -> 16 warps), N =
+// 512 x 4096 346 -> 258 and N = 128 x 16384 338 -> 267 (half of each warp idle).
+template <int L, int HB>
+__device__ __forceinline__ void dft_shared(const float2 (&lo)[L / 4], const float2 (&hi)[L / 4], int h,
+                                           float2 (&v)[L / 2]) {
+    constexpr int q = L / 4;
+    const float2 sgn = h ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
+    sfor<0, q>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        const float2 s = f2_add(lo[i], hi[i]);
+        float2 d = f2_sub(lo[i], hi[i]);
+        if constexpr (i == 0) {
+            d = h ? make_float2(d.y, -d.x) : d;  // W^q = -j, W^0 = 1
+        } else {
+            // W_L^(q h + i), as mul_w multiplies by it
+            constexpr float c0 = (float)cos2pi(i, L), s0 = (float)sin2pi(i, L);
+            constexpr float c1 = (float)cos2pi(q + i, L), s1 = (float)sin2pi(q + i, L);
+            const float c = h ? c1 : c0, sn = h ? s1 : s0;
+            d = make_float2(fmaf(d.x, c, d.y * sn), fmaf(d.y, c, -(d.x * sn)));
+        }
+        const float2 keep = h ? d : s, give = h ? s : d;
+        const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, HB), __shfl_xor_sync(0xffffffffu, give.y, HB));
+        v[i] = f2_add(keep, got);
+        v[i + q] = mul_w<i, L / 2>(f2_mul(f2_sub(keep, got), sgn));
+    });
+    fft_dif<L / 2, L / 2, 1>(v);
+}
+
 template <int N, bool I8, int MODE, int FEAT, int P = 0>
-__global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >= 512)) ? 1 : (N >= 512 ? 2 : 3)) k_fengine(const void *__restrict__ volt,
+__global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg<N, I8, MODE, FEAT>::NT == 512 ? 1 : 2)
+                                                               : (MODE == kPower && N >= 1024) ? 1 : (N >= 512 ? 2 : 3)) k_fengine(const void *__restrict__ volt,
                                                       const float *__restrict__ scale,
                                                       void *__restrict__ out,
                                                       double *__restrict__ power, int n_in, int K,
@@ -256,8 +303,11 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
                                                       const PfbArgs pfb) {
     using C = FCfg<N, I8, MODE, FEAT>;
     constexpr int T1 = C::T1, T2 = C::T2, TG = C::TG, G = C::G, EXS = C::EXS, SB = C::SB, ROWW = C::ROWW;
-    constexpr int TV = T1 > T2 ? T1 : T2;  // register values per thread
-    // square 32- or 64-point passes read the exchange into float arrays and do pass 2's
+    constexpr int NT = C::NT, H1 = C::H1, H2 = C::H2;
+    constexpr int R1 = T1 / H1, R2 = T2 / H2;  // values per thread in each pass
+    constexpr int TV = R1 > R2 ? R1 : R2;
+    constexpr int HB = T1 < 16 ? T1 : 16;      // lane bit between two threads that share a DFT
+    // square 32-point passes read the exchange into float arrays and do pass 2's
     // first stage in scalar arithmetic (no register moves into the (re, im) pairs); the
     // smaller lengths keep the in-place reads, which fit their register budgets
     constexpr bool kScalarStage = T1 == T2 && T2 >= 32;
@@ -282,7 +332,8 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
     };
     // the threads of one FFT group meet: a warp (or part of one), or the whole CTA
     auto group_sync = [] {
-        if constexpr (TG <= 32) __syncwarp(); else __syncthreads();
+        if constexpr (TG <= 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)threadIdx.x / TG), "n"(TG) : "memory");  // (warps of this group)
     };
 
     const int i = i0 + blockIdx.y;
@@ -321,7 +372,7 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
         if (hi > lo) {
             const char *blk = reinterpret_cast<const char *>(volt) + ((size_t)i * n_rec + lo) * BPS;
             const int lines = (int)(((hi - lo) * BPS + 127) / 128);
-            for (int l = threadIdx.x; l < lines; l += kThreads)
+            for (int l = threadIdx.x; l < lines; l += NT)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(blk + (size_t)l * 128));
         }
     }
@@ -329,10 +380,11 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
     // faster than L1 lookups, while the channel scales are faster from L1)
     const bool tw_async = PFB && !has_dly;  // as it stands: in flight while the first frames form
     if (tw_async) {
-        for (int m = 2 * threadIdx.x; m < N; m += 2 * kThreads) cp_async16(tws + m, tw_glob + m);
+        for (int m = 2 * threadIdx.x; m < N; m += 2 * NT) cp_async16(tws + m, tw_glob + m);
         cp_async_commit();
     }
-    for (int m = threadIdx.x; m < N && !tw_async; m += kThreads) {
+    if (C::TWG && has_dly && threadIdx.x < T2) dsm[threadIdx.x] = __ldg(dph + (size_t)i * (T1 + T2) + T1 + threadIdx.x);
+    for (int m = threadIdx.x; m < N && !tw_async && !C::TWG; m += NT) {
         float2 w = __ldg(tw_glob + m);
         if (DLY && has_dly) {
             w = cmul(w, __ldg(dph + (size_t)i * (T1 + T2) + m / T2));  // table [k1][t]: c[k1]
@@ -346,58 +398,70 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
 
     const int g = threadIdx.x / TG;
     const int t = threadIdx.x % TG;
-    // pass 1 uses threads t < T2 (the columns), pass 2 threads k1 = t < T1 (the rows)
-    const bool act1 = T2 == TG || t < T2, act2 = T1 == TG || t < T1;
+    // the column this thread takes in pass 1 and the row in pass 2, and which half of a
+    // shared DFT (the threads HB lanes apart)
+    const int half = (t / HB) & 1, pair = (t % HB) + (t / (2 * HB)) * HB;
+    const int col = H1 == 2 ? pair : t, row = H2 == 2 ? pair : t;
+    const int h1 = H1 == 2 ? half : 0, h2 = H2 == 2 ? half : 0;
     float *exg = ex + (size_t)g * C::GS;
-    const float4 *exrow = reinterpret_cast<const float4 *>(exg + (act2 ? t : 0) * EXS);
-    float pw[T2];
+    const float4 *exrow = reinterpret_cast<const float4 *>(exg + row * EXS);
+    float pw[R2];
     if constexpr (MODE == kPower) {
 #pragma unroll
-        for (int q = 0; q < T2; ++q) pw[q] = 0.0f;
+        for (int q = 0; q < R2; ++q) pw[q] = 0.0f;
     }
 
     for (int s0 = 0; s0 < SB; s0 += G) {
         const int s = s0 + g;
         const int a = a0 + s;
         const bool valid = (s < SB) && (a < K);
-        const bool valid1 = valid && act1;
         float2 v[TV];
-        // ---- pass 1: thread t takes x[t + T2 m]
+        // ---- pass 1: column col takes x[col + T2 m]: value m of the R1 this thread holds is
+        // sample mm(m) of the column
+        // twiddle W_N^(col k1) (with the delay phase c[k1]; / 256 for scaled samples)
+        auto tw_at = [&](int k1) {
+            if constexpr (!C::TWG) return tws[k1 * T2 + col];
+            float2 w = __ldg(tw_glob + k1 * T2 + col);
+            if (DLY && has_dly) w = cmul(w, __ldg(dph + (size_t)i * (T1 + T2) + k1));
+            if constexpr (SCALED) w = make_float2(w.x * (1.0f / kI8Scale), w.y * (1.0f / kI8Scale));
+            return w;
+        };
+        auto mm = [&](int m) { return H1 == 1 ? m : (m < R1 / 2 ? 0 : T1 / 2 - R1 / 2) + (T1 / 4) * h1 + m; };
         // sample offset of this frame in input i's stream (shifted by D with delays)
         const long long off = (long long)(valid ? a : 0) * N + D;
-        const long long base = (long long)i * n_rec + off + t;
+        const long long base = (long long)i * n_rec + off + col;
         // with delays, frames that reach outside the record take the checked loads
         const bool inside = !DLY || (off >= 0 && off + N <= n_rec);
         if constexpr (PFB) {
             if (s0 > 0) __syncthreads();  // every FFT has left its slot
-            pfb_frames<N, P, G, C::GS>(ex, reinterpret_cast<const char2 *>(volt) + (size_t)i * n_rec, pfb, D, n_rec,
+            pfb_frames<N, P, G, C::GS, NT>(ex, reinterpret_cast<const char2 *>(volt) + (size_t)i * n_rec, pfb, D, n_rec,
                                        a0 + s0);
             cp_async_wait_all();
             __syncthreads();
             const float2 *frame = reinterpret_cast<const float2 *>(exg);
 #pragma unroll
-            for (int m = 0; m < T1; ++m) v[m] = valid1 ? frame[pfb_at(t + T2 * m)] : make_float2(0.f, 0.f);
+            for (int m = 0; m < R1; ++m) v[m] = valid ? frame[pfb_at(col + T2 * mm(m))] : make_float2(0.f, 0.f);
             group_sync();  // read before the exchange overwrites the slot
         } else if constexpr (I8) {
             const unsigned short *src = reinterpret_cast<const unsigned short *>(volt) + base;
             if (use_async) {
                 cp_async_wait_all();
                 group_sync();  // every thread's pieces of the frame have landed
-                const unsigned short *raw = reinterpret_cast<const unsigned short *>(exg) + t;
+                const unsigned short *raw = reinterpret_cast<const unsigned short *>(exg) + col;
 #pragma unroll
-                for (int m = 0; m < T1; ++m) v[m] = i8_to_f2_scaled(valid1 ? (uint32_t)raw[T2 * m] : 0u);
+                for (int m = 0; m < R1; ++m) v[m] = i8_to_f2_scaled(valid ? (uint32_t)raw[T2 * mm(m)] : 0u);
                 group_sync();  // read before the exchange overwrites the buffer
             } else if (inside) {
 #pragma unroll
-                for (int m = 0; m < T1; ++m) {
-                    const uint32_t w = valid1 ? (uint32_t)__ldg(src + (size_t)T2 * m) : 0u;
+                for (int m = 0; m < R1; ++m) {
+                    const uint32_t w = valid ? (uint32_t)__ldg(src + (size_t)T2 * mm(m)) : 0u;
                     v[m] = SCALED ? i8_to_f2_scaled(w) : i8_to_f2(w);
                 }
             } else {
 #pragma unroll
-                for (int m = 0; m < T1; ++m) {
-                    const long long n = off + t + T2 * m;
-                    const uint32_t w = (valid1 && n >= 0 && n < n_rec) ? (uint32_t)__ldg(src + (long long)T2 * m) : 0u;
+                for (int m = 0; m < R1; ++m) {
+                    const long long n = off + col + T2 * mm(m);
+                    const uint32_t w = (valid && n >= 0 && n < n_rec) ? (uint32_t)__ldg(src + (long long)T2 * mm(m)) : 0u;
                     v[m] = SCALED ? i8_to_f2_scaled(w) : i8_to_f2(w);
                 }
             }
@@ -405,36 +469,73 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
             const float2 *src = reinterpret_cast<const float2 *>(volt) + base;
             if (inside) {
 #pragma unroll
-                for (int m = 0; m < T1; ++m) v[m] = valid1 ? __ldg(src + (size_t)T2 * m) : make_float2(0.f, 0.f);
+                for (int m = 0; m < R1; ++m) v[m] = valid ? __ldg(src + (size_t)T2 * mm(m)) : make_float2(0.f, 0.f);
             } else {
 #pragma unroll
-                for (int m = 0; m < T1; ++m) {
-                    const long long n = off + t + T2 * m;
-                    v[m] = (valid1 && n >= 0 && n < n_rec) ? __ldg(src + (long long)T2 * m) : make_float2(0.f, 0.f);
+                for (int m = 0; m < R1; ++m) {
+                    const long long n = off + col + T2 * mm(m);
+                    v[m] = (valid && n >= 0 && n < n_rec) ? __ldg(src + (long long)T2 * mm(m)) : make_float2(0.f, 0.f);
                 }
             }
         }
-        fft_dif<T1>(v);  // v[bitrev(k1)] = Y[t][k1] (x 256, bin 0 offset, for int8 input)
-        if constexpr (SCALED) v[0] = kOffsetFix<T1>(v[0]);
-        sfor<0, T1>([&](auto K1) {
+        // v[bitrev(k')] = Y[col][k1], k1 = H1 k' + h1 (x 256, bin 0 offset, for int8 input)
+        if constexpr (H1 == 1) {
+            fft_dif<T1>(v);
+        } else {
+            float2 lo[R1 / 2], hi[R1 / 2];
+#pragma unroll
+            for (int m = 0; m < R1 / 2; ++m) lo[m] = v[m], hi[m] = v[m + R1 / 2];
+            dft_shared<T1, HB>(lo, hi, h1, v);
+        }
+        if constexpr (SCALED) v[0] = h1 == 0 ? kOffsetFix<T1>(v[0]) : v[0];
+        sfor<0, R1>([&](auto K1) {
             constexpr int k1 = decltype(K1)::value;
-            // twiddle W_N^(t k1), table laid out [k1][t]
-            if constexpr (k1 != 0)
-                if (act1) v[bitrev(k1, ilog2(T1))] = cmul(v[bitrev(k1, ilog2(T1))], tws[k1 * T2 + t]);
+            // twiddle W_N^(col k1), table laid out [k1][col]
+            float2 &x = v[bitrev(k1, ilog2(R1))];
+            if constexpr (H1 == 1) {
+                if constexpr (k1 != 0) x = cmul(x, tw_at(k1));
+            } else {
+                const float2 y = cmul(x, tw_at(2 * k1 + h1));
+                x = k1 == 0 && h1 == 0 ? x : y;
+            }
         });
-        // ---- exchange (Re, then Im; the other half stays in place) and pass 2:
-        // thread t now plays k1 = t and takes Y[tt][k1], tt < T2
-        if (act1)
-            sfor<0, T1>([&](auto K1) {
-                constexpr int k1 = decltype(K1)::value;
-                exg[k1 * EXS + t] = v[bitrev(k1, ilog2(T1))].x;
-            });
+        // ---- exchange (Re, then Im; the other half stays in place) and pass 2: this thread
+        // now takes Y[tt][row]
+        sfor<0, R1>([&](auto K1) {
+            constexpr int k1 = decltype(K1)::value;
+            exg[(H1 * k1 + h1) * EXS + col] = v[bitrev(k1, ilog2(R1))].x;
+        });
         group_sync();
-        if constexpr (kScalarStage) {
+        if constexpr (H2 == 2) {
+            // tt = q h2 + i and T2 / 2 + q h2 + i, i < q
+            constexpr int q = T2 / 4;
+            float2 lo[q], hi[q];
+#pragma unroll
+            for (int j = 0; j < q / 4; ++j) {
+                const float4 a = exrow[q / 4 * h2 + j], b = exrow[T2 / 8 + q / 4 * h2 + j];
+                lo[4 * j].x = a.x, lo[4 * j + 1].x = a.y, lo[4 * j + 2].x = a.z, lo[4 * j + 3].x = a.w;
+                hi[4 * j].x = b.x, hi[4 * j + 1].x = b.y, hi[4 * j + 2].x = b.z, hi[4 * j + 3].x = b.w;
+            }
+            group_sync();
+            sfor<0, R1>([&](auto K1) {
+                constexpr int k1 = decltype(K1)::value;
+                exg[(H1 * k1 + h1) * EXS + col] = v[bitrev(k1, ilog2(R1))].y;
+            });
+            group_sync();
+#pragma unroll
+            for (int j = 0; j < q / 4; ++j) {
+                const float4 a = exrow[q / 4 * h2 + j], b = exrow[T2 / 8 + q / 4 * h2 + j];
+                lo[4 * j].y = a.x, lo[4 * j + 1].y = a.y, lo[4 * j + 2].y = a.z, lo[4 * j + 3].y = a.w;
+                hi[4 * j].y = b.x, hi[4 * j + 1].y = b.y, hi[4 * j + 2].y = b.z, hi[4 * j + 3].y = b.w;
+            }
+            group_sync();
+            if (use_async && s0 + G < SB) issue_raw(s0 + G + g);  // next frame into the free buffer
+            dft_shared<T2, HB>(lo, hi, h2, v);  // v[bitrev(k')] = X[row + T1 k2], k2 = 2 k' + h2
+        } else if constexpr (kScalarStage) {
             // the rows are read into plain float arrays (a 16-byte load fills four
             // consecutive registers, which the (re, im) register pairs of v cannot offer)
             float rin[T2], iin[T2];
-            if (act2) {
+            {
 #pragma unroll
                 for (int j = 0; j < T2 / 4; ++j) {
                     const float4 r = exrow[j];
@@ -442,13 +543,12 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
                 }
             }
             group_sync();
-            if (act1)
-                sfor<0, T1>([&](auto K1) {
-                    constexpr int k1 = decltype(K1)::value;
-                    exg[k1 * EXS + t] = v[bitrev(k1, ilog2(T1))].y;
-                });
+            sfor<0, T1>([&](auto K1) {
+                constexpr int k1 = decltype(K1)::value;
+                exg[k1 * EXS + t] = v[bitrev(k1, ilog2(T1))].y;
+            });
             group_sync();
-            if (act2) {
+            {
 #pragma unroll
                 for (int j = 0; j < T2 / 4; ++j) {
                     const float4 r = exrow[j];
@@ -470,7 +570,7 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
             });
             fft_dif<T2, TV, 1>(v);  // v[bitrev(k2)] = X[t + T1 k2]
         } else {
-            if (act2) {
+            {
 #pragma unroll
                 for (int j = 0; j < T2 / 4; ++j) {
                     const float4 r = exrow[j];
@@ -478,13 +578,12 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
                 }
             }
             group_sync();
-            if (act1)
-                sfor<0, T1>([&](auto K1) {
-                    constexpr int k1 = decltype(K1)::value;
-                    exg[k1 * EXS + t] = v[bitrev(k1, ilog2(T1))].y;
-                });
+            sfor<0, T1>([&](auto K1) {
+                constexpr int k1 = decltype(K1)::value;
+                exg[k1 * EXS + t] = v[bitrev(k1, ilog2(T1))].y;
+            });
             group_sync();
-            if (act2) {
+            {
 #pragma unroll
                 for (int j = 0; j < T2 / 4; ++j) {
                     const float4 r = exrow[j];
@@ -498,18 +597,21 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
         if (PFB && has_dly) {
             // delay phases exp(+j 2 pi T1 k2 f / N), in a block of their own: without delays
             // the plain filter bank skips it as a whole
-            sfor<1, T2>([&](auto K2) {
+            sfor<0, R2>([&](auto K2) {
                 constexpr int k2 = decltype(K2)::value;
-                v[bitrev(k2, ilog2(T2))] = cmul(v[bitrev(k2, ilog2(T2))], dsm[k2]);
+                float2 &x = v[bitrev(k2, ilog2(R2))];
+                const float2 y = cmul(x, dsm[H2 * k2 + h2]);
+                x = k2 == 0 && h2 == 0 ? x : y;
             });
         }
-        if (valid && act2) {
-            sfor<0, T2>([&](auto K2) {
+        if (valid) {
+            sfor<0, R2>([&](auto K2) {
                 constexpr int k2 = decltype(K2)::value;
-                const int k = t + T1 * k2;
-                float2 x = v[bitrev(k2, ilog2(T2))];
-                if constexpr (FEAT == kDelay && k2 != 0) {
-                    if (has_dly) x = cmul(x, dsm[k2]);  // delay phase exp(+j 2 pi T1 k2 f / N)
+                [[maybe_unused]] const int k = row + T1 * (H2 * k2 + h2);
+                float2 x = v[bitrev(k2, ilog2(R2))];
+                if constexpr (FEAT == kDelay && (k2 != 0 || H2 == 2)) {
+                    // delay phase exp(+j 2 pi T1 k2 f / N)
+                    if (has_dly && (k2 != 0 || h2 != 0)) x = cmul(x, dsm[H2 * k2 + h2]);
                 }
                 if constexpr (MODE == kRequant || MODE == kRequantPlanar) {
                     const uint32_t q = pack_q<MODE == kRequantPlanar>(x, __ldg(scale + k));
@@ -535,7 +637,7 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
                 // each thread moves 8 spectra of one channel row: 4 staged words
                 // (the code pairs of 2 spectra each) -> one 16-byte store per plane
                 constexpr int CPR = SB / 8;          // 8-spectrum chunks per row
-                constexpr int RPI = kThreads / CPR;  // rows per iteration
+                constexpr int RPI = NT / CPR;  // rows per iteration
                 const int q = threadIdx.x % CPR;
                 int k = threadIdx.x / CPR;
                 // physical words of logical words 4q .. 4q + 3 in row k; the swizzle
@@ -563,7 +665,7 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
             } else {
                 // unaligned rows or a short last block: a thread per code, whole rows per store
                 // instruction (one write request per row), U staged codes in flight
-                constexpr int U = 8, RPI = kThreads / SB;  // rows per round
+                constexpr int U = 8, RPI = NT / SB;  // rows per round
                 const uint16_t *sh = reinterpret_cast<const uint16_t *>(stg);
                 const size_t plane = (size_t)n_in * K;
                 const int c = threadIdx.x % SB;
@@ -589,7 +691,7 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
         } else {
             float2 *dst = reinterpret_cast<float2 *>(out);
             const float2 *sh = reinterpret_cast<const float2 *>(stg);
-            for (int e = threadIdx.x; e < N * SB; e += kThreads) {
+            for (int e = threadIdx.x; e < N * SB; e += NT) {
                 int k = e / SB, c = e % SB;
                 if (c < nv) dst[((size_t)k * n_in + i) * K + a0 + c] = sh[(size_t)k * (ROWW / 2) + c];
             }
@@ -597,13 +699,12 @@ __global__ void __launch_bounds__(kThreads, (N >= 2048 || (MODE == kPower && N >
     }
 
     if constexpr (MODE == kPower) {
-        if (act2)
-            sfor<0, T2>([&](auto K2) {
-                constexpr int k2 = decltype(K2)::value;
-                atomicAdd(&scs[t + T1 * k2], pw[k2]);
-            });
+        sfor<0, R2>([&](auto K2) {
+            constexpr int k2 = decltype(K2)::value;
+            atomicAdd(&scs[row + T1 * (H2 * k2 + h2)], pw[k2]);
+        });
         __syncthreads();
-        for (int m = threadIdx.x; m < N; m += kThreads) atomicAdd(&power[m], (double)scs[m]);
+        for (int m = threadIdx.x; m < N; m += NT) atomicAdd(&power[m], (double)scs[m]);
     }
 }
 
@@ -621,7 +722,7 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     // asynchronous raw copies need 16-byte aligned frames (2 N bytes each, N >= 64); the
     // public entry points only accept 16-byte aligned voltages, so this is a safeguard
     const int async_raw = reinterpret_cast<uintptr_t>(volt) % 16 == 0;
-    kern<<<grid, kThreads, C::smem, st>>>(volt, scale, out, power, f.n_in, f.n_spectra, f.tw, f.i0, vec_out,
+    kern<<<grid, C::NT, C::smem, st>>>(volt, scale, out, power, f.n_in, f.n_spectra, f.tw, f.i0, vec_out,
                                           f.dint, f.dph, async_raw, pfb);
     return check_launch("k_fengine");
 }
