@@ -573,22 +573,33 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
             const float *rs = p.rsc ? p.rsc + (long long)chan * p.n_in : nullptr;
             float si = 1.f;
             if (rs && i < (p.rect ? p.n_p : itm.n_in)) si = __ldg(rs + gi0 + i);
-#pragma unroll 1
-            for (int cb = 0; cb < 4; ++cb) {
+            // the tile's sums into registers first, so that the MMAs of the next tile wait for
+            // the reads only, not for the scaling and the writes below (plain FP16, 2048 inputs
+            // x 16 channels x 2048 spectra: 403 -> 379 us; hi/lo, three times the MMAs per
+            // tile, unchanged)
+            float V[64];  // Re of column 32 qc + x in V[x], Im in V[32 + x]
+#pragma unroll
+            for (int cb = 0; cb < 8; ++cb) {
                 // D1 = (re_I re_J | re_I im_J) in columns 0..255, D2 = (im_I re_J | im_I im_J) in 256..511
-                uint32_t a1[8], b2[8], a2[8], b1[8];
-                tc::tmem_ld8(d + 8u * cb, a1);
-                tc::tmem_ld8(d + 384u + 8u * cb, b2);
-                tc::tmem_ld8(d + 256u + 8u * cb, a2);
-                tc::tmem_ld8(d + 128u + 8u * cb, b1);
+                uint32_t u[8], w[8];
+                tc::tmem_ld8(d + 8u * (cb & 3) + (cb < 4 ? 0u : 256u), u);
+                tc::tmem_ld8(d + 8u * (cb & 3) + (cb < 4 ? 384u : 128u), w);
                 tc::tmem_wait_ld();
+#pragma unroll
+                for (int x = 0; x < 8; ++x)
+                    V[8 * cb + x] = cb < 4 ? __uint_as_float(u[x]) + __uint_as_float(w[x])
+                                           : __uint_as_float(u[x]) - __uint_as_float(w[x]);
+            }
+            tc::tc_fence_before();
+            tc::mbar_arrive(acce_bar(0));
+#pragma unroll
+            for (int cb = 0; cb < 4; ++cb) {
                 const int jb = J0 + 32 * qc + 8 * cb;  // columns jb .. jb + 7
                 // row `lane`, column x at element lane * 8 + ((x + lane / 2) & 7): two
                 // wavefronts per 8-byte store of one x and per 4-row read below
 #pragma unroll
                 for (int x = 0; x < 8; ++x) {
-                    float2 v = make_float2(__uint_as_float(a1[x]) + __uint_as_float(b2[x]),
-                                           __uint_as_float(a2[x]) - __uint_as_float(b1[x]));
+                    float2 v = make_float2(V[8 * cb + x], V[32 + 8 * cb + x]);
                     const int jg = min(jb + x, (p.rect ? p.n_q : itm.n_in) - 1);  // clamped: unused past the end
                     if (rs) {
                         const float sij = si * __ldg(rs + gj0 + jg);
@@ -603,50 +614,47 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
                 }
                 __syncwarp();
                 // offsets within the channel's block (below 2^32 entries: one channel's
-                // triangle or rectangle)
-                float2 val[8];
-                uint32_t off[8];
-                bool ok[8];
+                // triangle or rectangle); four rows at a time, every read of a
+                // read-modify-write in flight before its writes
+#pragma unroll 1
+                for (int h4 = 0; h4 < 8; h4 += 4) {
+                    float2 val[4];
+                    uint32_t off[4];
+                    bool ok[4];
 #pragma unroll
-                for (int rr = 0; rr < 8; ++rr) {
-                    const int r = rr * 4 + (lane >> 3), e = lane & 7;
-                    const int ii = I0 + wq * 32 + r, jj = jb + e;
-                    val[rr] = sl[r * 8 + ((e + (r >> 1)) & 7)];
-                    ok[rr] = p.rect ? (ii < p.n_p && jj < p.n_q) : (ii < itm.n_in && jj <= ii);
-                    off[rr] = p.rect ? (uint32_t)ii * (uint32_t)p.n_q + jj
-                                     : (uint32_t)(((unsigned long long)ii * (unsigned)(ii + 1)) >> 1) + jj;
-                }
-                __syncwarp();
-                // read-modify-writes: every read of a round in flight before its writes
-                if (p.vis64) {
-                    double2 *dst = p.vis64 + (long long)chan * itm.B;
-#pragma unroll
-                    for (int h4 = 0; h4 < 8; h4 += 4) {
+                    for (int q = 0; q < 4; ++q) {
+                        const int r = (h4 + q) * 4 + (lane >> 3), e = lane & 7;
+                        const int ii = I0 + wq * 32 + r, jj = jb + e;
+                        val[q] = sl[r * 8 + ((e + (r >> 1)) & 7)];
+                        ok[q] = p.rect ? (ii < p.n_p && jj < p.n_q) : (ii < itm.n_in && jj <= ii);
+                        off[q] = p.rect ? (uint32_t)ii * (uint32_t)p.n_q + jj
+                                        : (uint32_t)(((unsigned long long)ii * (unsigned)(ii + 1)) >> 1) + jj;
+                    }
+                    if (p.vis64) {
+                        double2 *dst = p.vis64 + (long long)chan * itm.B;
                         double2 o[4];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) o[q] = ok[h4 + q] ? __ldcg(dst + off[h4 + q]) : make_double2(0.0, 0.0);
+                        for (int q = 0; q < 4; ++q) o[q] = ok[q] ? __ldcg(dst + off[q]) : make_double2(0.0, 0.0);
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            if (ok[h4 + q])
-                                dst[off[h4 + q]] = add_exact(o[q], val[h4 + q]);  // FP32 sums: conversion in integers
+                            if (ok[q]) dst[off[q]] = add_exact(o[q], val[q]);  // FP32 sums: conversion in integers
+                    } else {
+                        float2 *dst = p.rect ? static_cast<float2 *>(p.rect_out) + (long long)chan * p.n_p * p.n_q
+                                             : static_cast<float2 *>(itm.acc) + (long long)chan * itm.B;
+                        if (!p.store) {
+                            float2 o[4];
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) o[q] = ok[q] ? __ldcg(dst + off[q]) : make_float2(0.f, 0.f);
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) val[q] = make_float2(val[q].x + o[q].x, val[q].y + o[q].y);
+                        }
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            if (ok[q]) dst[off[q]] = val[q];
                     }
-                } else {
-                    float2 *dst = p.rect ? static_cast<float2 *>(p.rect_out) + (long long)chan * p.n_p * p.n_q
-                                         : static_cast<float2 *>(itm.acc) + (long long)chan * itm.B;
-                    if (!p.store) {
-                        float2 o[8];
-#pragma unroll
-                        for (int rr = 0; rr < 8; ++rr) o[rr] = ok[rr] ? __ldcg(dst + off[rr]) : make_float2(0.f, 0.f);
-#pragma unroll
-                        for (int rr = 0; rr < 8; ++rr) val[rr] = make_float2(val[rr].x + o[rr].x, val[rr].y + o[rr].y);
-                    }
-#pragma unroll
-                    for (int rr = 0; rr < 8; ++rr)
-                        if (ok[rr]) dst[off[rr]] = val[rr];
                 }
+                __syncwarp();
             }
-            tc::tc_fence_before();
-            tc::mbar_arrive(acce_bar(0));
         }
     } else if (W && warp >= 4) {
         // ------------------------------------------------------------ wide INT8 epilogue
