@@ -18,6 +18,7 @@ corr_status dispatch(const FShape &f, const void *volt, const float *scale, void
 
 FShape shape_of(const Handle &h) {
     FShape f{h.n_in, h.n_chan, h.n_spectra, h.precision == CORR_PREC_INT8, h.twiddle};
+    f.n_sm = h.n_sm;
     if (h.dly_int) {
         f.dint = h.dly_int;
         f.dph = h.dly_ph;

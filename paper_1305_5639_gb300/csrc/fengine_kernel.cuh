@@ -46,6 +46,7 @@ struct FShape {
     int i0 = 0, n_run = -1;  // inputs [i0, i0 + n_run) of the n_in (n_run < 0: all)
     const int *dint = nullptr;     // per-input integer advance (delay compensation), or null
     const float2 *dph = nullptr;   // per-input phase tables [n_in][T1 + T2]: c[k1], then d[k2]
+    int n_sm = 152;
 };
 
 namespace {
@@ -96,6 +97,9 @@ struct FCfg {
     static constexpr int SB = MODE == kFloatOut ? (N <= 1024 ? (G > 8 ? G : 8) : 8192 / N)
                                                 : (RQ ? (FEAT == kPfb && N == 1024 ? 16 : N <= 1024 ? 32 : (N == 4096 && FEAT != kPfb) ? 16 : 32768 / N)
                                                       : (G > 16 ? G : 16));
+    // The long transforms may take fewer spectra per CTA than SB (see launch_one_); for the
+    // others the variable loop bound cost more (1 to 4 %) than a fuller chip gains.
+    static constexpr bool VARSB = RQ && N >= 2048;
     // staging row stride in 32-bit words. The re-packing modes stage one 16-bit code
     // pair per (channel k, spectrum s): a row of SB / 2 words whose word index is
     // XOR-swizzled with (k >> SW) & (ROWW - 1), SW = log2(32 / ROWW), so that the
@@ -300,7 +304,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
                                                       const float2 *__restrict__ tw_glob, int i0, int vec_out,
                                                       const int *__restrict__ dint,
                                                       const float2 *__restrict__ dph, int async_raw,
-                                                      const PfbArgs pfb) {
+                                                      const PfbArgs pfb, int sb_run) {
     using C = FCfg<N, I8, MODE, FEAT>;
     constexpr int T1 = C::T1, T2 = C::T2, TG = C::TG, G = C::G, EXS = C::EXS, SB = C::SB, ROWW = C::ROWW;
     constexpr int NT = C::NT, H1 = C::H1, H2 = C::H2;
@@ -337,7 +341,8 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
     };
 
     const int i = i0 + blockIdx.y;
-    const int a0 = blockIdx.x * SB;
+    const int sb = C::VARSB ? sb_run : SB;  // spectra per CTA
+    const int a0 = blockIdx.x * sb;
     // Raw int8 frames without delays are copied asynchronously into the FFT's exchange
     // buffer (free between exchanges): the copy for the next frame is issued after the
     // current frame's exchange and lands while its pass 2 and re-packing run. Each of
@@ -348,7 +353,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
     // copy of frame s_ of this CTA into the exchange buffer of FFT slot s_ % G
     auto issue_raw = [&](int s_) {
         const int a_ = a0 + s_, t_ = threadIdx.x % TG;
-        if (s_ < SB && a_ < K) {
+        if (s_ < sb && a_ < K) {
             const char *src = reinterpret_cast<const char *>(volt) + ((size_t)i * K + a_) * (size_t)N * 2;
             char *dst = reinterpret_cast<char *>(ex + (size_t)(s_ % G) * C::GS);
 #pragma unroll
@@ -368,7 +373,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
         // contiguous range): the loads of the later spectra then hit L2 instead of HBM.
         constexpr int BPS = I8 ? 2 : 8;  // bytes per complex sample
         const long long lo = max(0LL, (long long)a0 * N + D);
-        const long long hi = min(n_rec, (long long)min(K, a0 + SB) * N + D);
+        const long long hi = min(n_rec, (long long)min(K, a0 + sb) * N + D);
         if (hi > lo) {
             const char *blk = reinterpret_cast<const char *>(volt) + ((size_t)i * n_rec + lo) * BPS;
             const int lines = (int)(((hi - lo) * BPS + 127) / 128);
@@ -412,6 +417,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
     }
 
     for (int s0 = 0; s0 < SB; s0 += G) {
+        if (C::VARSB && s0 >= sb) break;  // (sb is a multiple of G)
         const int s = s0 + g;
         const int a = a0 + s;
         const bool valid = (s < SB) && (a < K);
@@ -529,7 +535,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
                 hi[4 * j].y = b.x, hi[4 * j + 1].y = b.y, hi[4 * j + 2].y = b.z, hi[4 * j + 3].y = b.w;
             }
             group_sync();
-            if (use_async && s0 + G < SB) issue_raw(s0 + G + g);  // next frame into the free buffer
+            if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
             dft_shared<T2, HB>(lo, hi, h2, v);  // v[bitrev(k')] = X[row + T1 k2], k2 = 2 k' + h2
         } else if constexpr (kScalarStage) {
             // the rows are read into plain float arrays (a 16-byte load fills four
@@ -556,7 +562,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
                 }
             }
             group_sync();
-            if (use_async && s0 + G < SB) issue_raw(s0 + G + g);  // next frame into the free buffer
+            if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
             // pass 2: its first radix-2 stage in scalar arithmetic, from the float arrays
             // into the (re, im) pairs, then the remaining stages on the pairs
             sfor<0, T2 / 2>([&](auto J) {
@@ -591,7 +597,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
                 }
             }
             group_sync();
-            if (use_async && s0 + G < SB) issue_raw(s0 + G + g);  // next frame into the free buffer
+            if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
             fft_dif<T2>(v);  // v[bitrev(k2)] = X[t + T1 k2]
         }
         if (PFB && has_dly) {
@@ -628,12 +634,12 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
     if constexpr (MODE != kPower) {
         __syncthreads();
         // ---- corner turn: row (k, i) gets spectra a0 .. a0 + nv - 1
-        const int nv = min(SB, K - a0);
+        const int nv = min(sb, K - a0);
         if constexpr (MODE == kRequantPlanar || MODE == kRequant) {
             uint16_t *dst = reinterpret_cast<uint16_t *>(out);
             // planar FP16 layout [k][plane][i][a]; int8 layout [k][i][a] (complex int8)
             constexpr int PL = MODE == kRequantPlanar ? 2 : 1;
-            if (nv == SB && vec_out) {
+            if (vec_out && (C::VARSB || nv == SB)) {  // nv is a multiple of 8: sb and K are
                 // each thread moves 8 spectra of one channel row: 4 staged words
                 // (the code pairs of 2 spectra each) -> one 16-byte store per plane
                 constexpr int CPR = SB / 8;          // 8-spectrum chunks per row
@@ -648,7 +654,8 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
                 const uint32_t *src = stg + (size_t)k * ROWW;
                 uint4 *d = reinterpret_cast<uint4 *>(dst + ((size_t)(PL * k) * n_in + i) * K + a0 + 8 * q);
                 const size_t dstep = (size_t)PL * RPI * n_in * K / 8, dplane = (size_t)n_in * K / 8;
-                for (; k < N; k += RPI, src += RPI * ROWW, d += dstep) {
+                const int k_end = !C::VARSB || 8 * q < nv ? N : 0;
+                for (; k < k_end; k += RPI, src += RPI * ROWW, d += dstep) {
                     const uint32_t w0 = src[o0], w1 = src[o1], w2 = src[o2], w3 = src[o3];
                     if constexpr (MODE == kRequantPlanar) {
                         uint4 re, im;
@@ -718,12 +725,20 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     const int vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0) && (f.n_spectra % 8 == 0);
     // blockIdx.x (the spectra block) varies fastest, so the CTAs resident at one time
     // write neighbouring segments of the same output rows
-    dim3 grid((f.n_spectra + C::SB - 1) / C::SB, f.n_run < 0 ? f.n_in : f.n_run);
+    // spectra per CTA: SB, or half or a quarter of it (whole rounds of the G FFTs in flight,
+    // whole 16-byte pieces of a row) while the launch has fewer CTAs than the chip has SMs:
+    // few inputs and spectra then take the time of one round instead of SB / G of them (7
+    // inputs x 80 spectra at N = 4096, one launch per input: 487 -> 396 us
+    // for the host pipeline's call)
+    const int n_rows = f.n_run < 0 ? f.n_in : f.n_run;
+    int sb = C::SB;
+    while (C::VARSB && sb / 2 >= C::G && sb / 2 >= 8 && (long long)((f.n_spectra + sb - 1) / sb) * n_rows < f.n_sm) sb /= 2;
+    dim3 grid((f.n_spectra + sb - 1) / sb, n_rows);
     // asynchronous raw copies need 16-byte aligned frames (2 N bytes each, N >= 64); the
     // public entry points only accept 16-byte aligned voltages, so this is a safeguard
     const int async_raw = reinterpret_cast<uintptr_t>(volt) % 16 == 0;
     kern<<<grid, C::NT, C::smem, st>>>(volt, scale, out, power, f.n_in, f.n_spectra, f.tw, f.i0, vec_out,
-                                          f.dint, f.dph, async_raw, pfb);
+                                          f.dint, f.dph, async_raw, pfb, sb);
     return check_launch("k_fengine");
 }
 
