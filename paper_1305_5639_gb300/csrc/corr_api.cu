@@ -168,7 +168,7 @@ bool use_tc(const Handle &h) {
 // replayed as they are issued.
 bool defer_ok(const Handle &h) {
     return (h.precision == CORR_PREC_INT8 || h.precision == CORR_PREC_FP16_HILO) && use_tc(h) &&
-           !(h.flags & CORR_FLAG_FUSED_DUMP) && tma_available();
+           !(h.flags & CORR_FLAG_FUSED_DUMP) && tma_available() && !xengine_i8_small(h);
 }
 
 // Remembers whether any call was recorded into a graph.
@@ -630,7 +630,7 @@ corr_status corr_xengine(corr_t *c, const void *chan_in, const float *gains, voi
     cudaStream_t st = corr::as_stream(stream);
     corr::note_capture(h, st);
     if (h.dump_pending || (h.flags & CORR_FLAG_FUSED_DUMP)) h.vis_zero = false;
-    if (corr::use_tc(h)) {
+    if (corr::use_tc(h) && !corr::xengine_i8_small(h)) {
         corr::TcOperands op;
         s = corr::tc_operands(h, chan_in, st, op);
         // a deferred dump of the previous integration rides along in this launch

@@ -124,6 +124,8 @@ corr_status launch_fengine(const Handle &h, const void *volt, const float *scale
 corr_status launch_fengine_power(const Handle &h, const void *volt, float *power, cudaStream_t st);
 corr_status launch_xengine_cudacore(const Handle &h, const void *chan_in, const float2 *gains,
                                     bool store, cudaStream_t st);
+// Whether an AUTO INT8 X-engine call runs on the CUDA cores: complex int8 layout, few inputs.
+bool xengine_i8_small(const Handle &h);
 corr_status launch_dump(const Handle &h, cudaStream_t st);
 corr_status launch_dump_range(const Handle &h, int c0, int c1, cudaStream_t st);
 // The dump of an accumulator other than the handle's current one (a deferred dump).

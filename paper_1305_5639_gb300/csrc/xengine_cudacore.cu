@@ -150,74 +150,25 @@ int f32_tile_ct(const Handle &h) {
     return best;
 }
 
-// Few inputs (n_in <= kSmallIn): one CTA per channel, one warp per 4 x 4 block of the
-// lower triangle and per K range (n_split of them), one lane per pair of spectra (per
-// spectrum where K is odd), so that the rows are read straight from global memory, 512
-// contiguous bytes per warp and row, and every load feeds four products. The 32 sums of a
-// block (16 pairs, Re and Im) are then added over the lanes by a transposing butterfly
-// that leaves sum number `lane` in each lane, and over the K ranges in order: a fixed
-// order, so the result is run-to-run identical. Bound by the L1 reads (each row is read
-// by the n_in / 4 + 1 blocks it meets) and the FP32 pipe: 14.5 us for 16 inputs, 256
+// Few inputs (n_in <= kSmallIn): one CTA per channel; a task is a 4 x 4 block of the lower
+// triangle over one K range (n_split of them), done by one warp with a lane per pair of
+// spectra (per spectrum where K is odd), so that the rows are read straight from global
+// memory, 512 contiguous bytes per warp and row, and every load feeds four products. The 32
+// sums of a block (16 pairs, Re and Im) are then added over the lanes by a transposing
+// butterfly that leaves sum number `lane` in each lane, and over the K ranges in order: a
+// fixed order, so the result is run-to-run identical. Bound by the L1 reads (each row is
+// read by the n_in / 4 + 1 blocks it meets) and the FP32 pipe: 14.5 us for 16 inputs, 256
 // channels, 1024 spectra (33.5 MB: 5 us of HBM time), against 30.4 us with one thread per
-// pair reading both factors of each product from shared memory. Above 22 inputs the 32-
-// and 48-input tiles of k_xeng_f32 have the better ratio of sums to reads.
-constexpr int kSmallIn = 22;
-constexpr int kSmallWarps = 21;  // 21 blocks at 22 inputs, else up to 20 warps
+// pair reading both factors of each product from shared memory. Above 32 inputs the tiles
+// of k_xeng_f32 have the better ratio of sums to reads (24 inputs, 256 channels, 1024
+// spectra: 35 us here, 60 us there).
+constexpr int kSmallIn = 32;     // at most 36 blocks
+constexpr int kSmallWarps = 20;
+constexpr int kSmallTasks = 36;  // blocks x K ranges
 
-template <bool VEC>
-__global__ void __launch_bounds__(32 * kSmallWarps) k_xeng_f32_small(const float2 *__restrict__ X, float2 *__restrict__ acc,
-                                                         const float2 *__restrict__ gains, int n_in, int K,
-                                                         long long B, int n_blk, int n_split, int store) {
-    __shared__ float part[kSmallWarps][32];
-    const int chan = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int blk = warp % n_blk, sp = warp / n_blk;
-    int bi, bj;
-    tile_of(blk, bi, bj);
-    const float2 *Xc = X + (size_t)chan * n_in * K;
-    // rows past the end read the last one; their sums are not written
-    const float2 *xi[4], *xj[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        xi[r] = Xc + (size_t)min(4 * bi + r, n_in - 1) * K;
-        xj[r] = Xc + (size_t)min(4 * bj + r, n_in - 1) * K;
-    }
-    float v[32];  // sum 2 (4 r + c) + part of pair (4 bi + r, 4 bj + c)
-#pragma unroll
-    for (int e = 0; e < 32; ++e) v[e] = 0.f;
-    auto mac = [&](const float2 (&a)[4], const float2 (&b)[4]) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                // x_i conj(x_j)
-                const int e = 2 * (4 * r + c);
-                v[e] = fmaf(a[r].x, b[c].x, fmaf(a[r].y, b[c].y, v[e]));
-                v[e + 1] = fmaf(a[r].y, b[c].x, fmaf(-a[r].x, b[c].y, v[e + 1]));
-            }
-    };
-    const int step = VEC ? 64 : 32;
-    for (int a = sp * step + (VEC ? 2 * lane : lane); a < K; a += n_split * step) {
-        if (VEC) {
-            float2 i0[4], i1[4], j0[4], j1[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float4 q = __ldg(reinterpret_cast<const float4 *>(xi[r] + a));
-                i0[r] = make_float2(q.x, q.y), i1[r] = make_float2(q.z, q.w);
-            }
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const float4 q = __ldg(reinterpret_cast<const float4 *>(xj[r] + a));
-                j0[r] = make_float2(q.x, q.y), j1[r] = make_float2(q.z, q.w);
-            }
-            mac(i0, j0);
-            mac(i1, j1);
-        } else {
-            float2 i0[4], j0[4];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) i0[r] = __ldg(xi[r] + a), j0[r] = __ldg(xj[r] + a);
-            mac(i0, j0);
-        }
-    }
+// the sums v[k] of all lanes: afterwards v[0] holds sum number `lane`
+template <typename T>
+__device__ __forceinline__ void butterfly32(T (&v)[32], int lane) {
     // after the step of width o, v[k] holds the sum over the lanes differing in bit o of
     // sum k (+ o for lanes with that bit set)
 #pragma unroll
@@ -226,26 +177,88 @@ __global__ void __launch_bounds__(32 * kSmallWarps) k_xeng_f32_small(const float
         for (int k = 0; k < 16; ++k) {
             if (k >= o) break;
             const bool up = (lane & o) != 0;
-            const float send = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
+            const T send = up ? v[k] : v[k + o], keep = up ? v[k + o] : v[k];
             v[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
     }
-    part[warp][lane] = v[0];
-    __syncthreads();
-    if (sp != 0) return;
-    float s = part[warp][lane];
-    for (int q = 1; q < n_split; ++q) s += part[warp + q * n_blk][lane];
-    const float other = __shfl_xor_sync(0xffffffffu, s, 1);
-    const int i = 4 * bi + (lane >> 3), j = 4 * bj + ((lane >> 1) & 3);
-    if ((lane & 1) || i >= n_in || j > i) return;
-    float2 w = make_float2(s, other);
-    if (gains) w = apply_gains(w, __ldg(gains + i), __ldg(gains + j));
-    const size_t b = (size_t)chan * B + (size_t)i * (i + 1) / 2 + j;
-    if (!store) {
-        const float2 o = acc[b];
-        w = make_float2(o.x + w.x, o.y + w.y);
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(32 * kSmallWarps) k_xeng_f32_small(const float2 *__restrict__ X, float2 *__restrict__ acc,
+                                                         const float2 *__restrict__ gains, int n_in, int K,
+                                                         long long B, int n_blk, int n_split, int store) {
+    __shared__ float part[kSmallTasks][32];
+    const int chan = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
+    const float2 *Xc = X + (size_t)chan * n_in * K;
+    const int step = VEC ? 64 : 32;
+#pragma unroll 1
+    for (int task = warp; task < n_blk * n_split; task += n_warp) {
+        int bi, bj;
+        tile_of(task % n_blk, bi, bj);
+        // rows past the end read the last one; their sums are not written
+        const float2 *xi[4], *xj[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            xi[r] = Xc + (size_t)min(4 * bi + r, n_in - 1) * K;
+            xj[r] = Xc + (size_t)min(4 * bj + r, n_in - 1) * K;
+        }
+        float v[32];  // sum 2 (4 r + c) + part of pair (4 bi + r, 4 bj + c)
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = 0.f;
+        auto mac = [&](const float2 (&a)[4], const float2 (&b)[4]) {
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    // x_i conj(x_j)
+                    const int e = 2 * (4 * r + c);
+                    v[e] = fmaf(a[r].x, b[c].x, fmaf(a[r].y, b[c].y, v[e]));
+                    v[e + 1] = fmaf(a[r].y, b[c].x, fmaf(-a[r].x, b[c].y, v[e + 1]));
+                }
+        };
+        for (int a = (task / n_blk) * step + (VEC ? 2 * lane : lane); a < K; a += n_split * step) {
+            if (VEC) {
+                float2 i0[4], i1[4], j0[4], j1[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float4 q = __ldg(reinterpret_cast<const float4 *>(xi[r] + a));
+                    i0[r] = make_float2(q.x, q.y), i1[r] = make_float2(q.z, q.w);
+                }
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const float4 q = __ldg(reinterpret_cast<const float4 *>(xj[r] + a));
+                    j0[r] = make_float2(q.x, q.y), j1[r] = make_float2(q.z, q.w);
+                }
+                mac(i0, j0);
+                mac(i1, j1);
+            } else {
+                float2 i0[4], j0[4];
+#pragma unroll
+                for (int r = 0; r < 4; ++r) i0[r] = __ldg(xi[r] + a), j0[r] = __ldg(xj[r] + a);
+                mac(i0, j0);
+            }
+        }
+        butterfly32(v, lane);
+        part[task][lane] = v[0];
     }
-    acc[b] = w;
+    __syncthreads();
+    for (int blk = warp; blk < n_blk; blk += n_warp) {
+        int bi, bj;
+        tile_of(blk, bi, bj);
+        float s = part[blk][lane];
+        for (int q = 1; q < n_split; ++q) s += part[blk + q * n_blk][lane];
+        const float other = __shfl_xor_sync(0xffffffffu, s, 1);
+        const int i = 4 * bi + (lane >> 3), j = 4 * bj + ((lane >> 1) & 3);
+        if ((lane & 1) || i >= n_in || j > i) continue;
+        float2 w = make_float2(s, other);
+        if (gains) w = apply_gains(w, __ldg(gains + i), __ldg(gains + j));
+        const size_t b = (size_t)chan * B + (size_t)i * (i + 1) / 2 + j;
+        if (!store) {
+            const float2 o = acc[b];
+            w = make_float2(o.x + w.x, o.y + w.y);
+        }
+        acc[b] = w;
+    }
 }
 
 __device__ __forceinline__ uint32_t rot_word(uint32_t w) {
@@ -255,6 +268,91 @@ __device__ __forceinline__ uint32_t rot_word(uint32_t w) {
 }
 // dp4a weights picking the imaginary bytes of a word: [0 1 0 1]
 constexpr int kImOnes = 0x01000100;
+
+// INT8 with few inputs (n_in <= kSmallIn), as k_xeng_f32_small: a lane takes W words of two
+// spectra per row and step (W = 4 where a row is whole 16-byte pieces, 1 for an even K; W = 0:
+// single spectra), every word feeding four dp4a pairs. Reads the complex int8 layout
+// directly, where the tensor cores need a conversion pass and spend a 128 x 128 tile on the
+// few pairs. X-engine and dump, tensor cores -> here (us): 16 inputs, 256 channels, 1024
+// spectra 39 -> 15; 8 inputs, 1024 channels, 512 spectra 70 -> 15; 32 inputs, 1024 channels,
+// 4096 spectra 471 -> 245.
+template <int W>
+__global__ void __launch_bounds__(32 * kSmallWarps) k_xeng_i8_small(const char2 *__restrict__ X, int2 *__restrict__ acc,
+                                                                    int n_in, int K, long long B, int n_blk,
+                                                                    int n_split, int store) {
+    __shared__ int part[kSmallTasks][32];
+    const int chan = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warp = blockDim.x >> 5;
+    const char2 *Xc = X + (size_t)chan * n_in * K;
+    constexpr int NW = W ? W : 1, S = W ? 2 * W : 1;  // words and spectra per lane and step
+#pragma unroll 1
+    for (int task = warp; task < n_blk * n_split; task += n_warp) {
+        int bi, bj;
+        tile_of(task % n_blk, bi, bj);
+        const char2 *xi[4], *xj[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            xi[r] = Xc + (size_t)min(4 * bi + r, n_in - 1) * K;
+            xj[r] = Xc + (size_t)min(4 * bj + r, n_in - 1) * K;
+        }
+        int v[32], cim[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = 0;
+        auto load = [](const char2 *p, uint32_t (&w)[NW]) {
+            if constexpr (W == 4) {
+                const uint4 q = __ldg(reinterpret_cast<const uint4 *>(p));
+                w[0] = q.x, w[1] = q.y, w[2] = q.z, w[3] = q.w;
+            } else if constexpr (W == 1) {
+                w[0] = __ldg(reinterpret_cast<const unsigned int *>(p));
+            } else {
+                w[0] = __ldg(reinterpret_cast<const unsigned short *>(p));
+            }
+        };
+        for (int a = ((task / n_blk) * 32 + lane) * S; a < K; a += n_split * 32 * S) {
+            uint32_t wi[4][NW], wj[4][NW];
+#pragma unroll
+            for (int r = 0; r < 4; ++r) load(xi[r] + a, wi[r]);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) load(xj[r] + a, wj[r]);
+#pragma unroll
+            for (int q = 0; q < NW; ++q) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) cim[c] = __dp4a((int)wj[c][q], kImOnes, cim[c]);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    // (a zero upper half rotates to (0, ~0): ~0 times the zero of x_j)
+                    const int x = (int)wi[r][q], rx = (int)rot_word(wi[r][q]);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const int e = 2 * (4 * r + c);
+                        v[e] = __dp4a(x, (int)wj[c][q], v[e]);
+                        v[e + 1] = __dp4a(rx, (int)wj[c][q], v[e + 1]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[2 * e + 1] += cim[e & 3];
+        butterfly32(v, lane);
+        part[task][lane] = v[0];
+    }
+    __syncthreads();
+    for (int blk = warp; blk < n_blk; blk += n_warp) {
+        int bi, bj;
+        tile_of(blk, bi, bj);
+        int s = part[blk][lane];
+        for (int q = 1; q < n_split; ++q) s += part[blk + q * n_blk][lane];
+        const int other = __shfl_xor_sync(0xffffffffu, s, 1);
+        const int i = 4 * bi + (lane >> 3), j = 4 * bj + ((lane >> 1) & 3);
+        if ((lane & 1) || i >= n_in || j > i) continue;
+        int2 w = make_int2(s, other);
+        const size_t b = (size_t)chan * B + (size_t)i * (i + 1) / 2 + j;
+        if (!store) {
+            const int2 o = acc[b];
+            w = make_int2(o.x + w.x, o.y + w.y);
+        }
+        acc[b] = w;
+    }
+}
 
 __global__ void __launch_bounds__(NTH) k_xeng_i8(const char2 *__restrict__ X, int2 *__restrict__ acc,
                                                  int n_in, int K, long long B, int store) {
@@ -347,23 +445,40 @@ __global__ void __launch_bounds__(NTH) k_xeng_i8(const char2 *__restrict__ X, in
 
 }  // namespace
 
+bool xengine_i8_small(const Handle &h) {
+    // (an odd number of spectra leaves single-spectrum loads: 32 inputs, 1024 channels, 1001
+    // spectra take 193 us here, 135 on the tensor cores; the work falls with the pairs)
+    return h.precision == CORR_PREC_INT8 && h.xengine == CORR_XENG_AUTO &&
+           h.n_in <= (h.n_spectra % 2 == 0 ? kSmallIn : 24) && !(h.flags & (CORR_FLAG_PLANAR | CORR_FLAG_FUSED_DUMP));
+}
+
 corr_status launch_xengine_cudacore(const Handle &h, const void *chan_in, const float2 *gains, bool store,
                                     cudaStream_t st) {
     StageScope sc(h, CORR_STAGE_XENGINE, st);
     corr_status s = CORR_OK;
     const float2 *X = static_cast<const float2 *>(chan_in);
-    if (h.precision == CORR_PREC_INT8) {
+    if (h.n_in <= kSmallIn) {
+        const int nb = (h.n_in + 3) / 4, n_blk = nb * (nb + 1) / 2;
+        const bool i8 = h.precision == CORR_PREC_INT8;
+        const int W = !i8 ? 0 : h.n_spectra % 8 == 0 ? 4 : h.n_spectra % 2 == 0 ? 1 : 0;
+        // K ranges: as many tasks as warps, as long as each range has a few rounds
+        const int round = i8 ? 32 * (W ? 2 * W : 1) : 64;
+        const int n_split = std::max(1, std::min(kSmallWarps / n_blk, h.n_spectra / (4 * round)));
+        const int threads = 32 * std::min(kSmallWarps, n_blk * n_split);
+        if (i8) {
+            auto kern = W == 4 ? k_xeng_i8_small<4> : W == 1 ? k_xeng_i8_small<1> : k_xeng_i8_small<0>;
+            kern<<<h.n_chan, threads, 0, st>>>(static_cast<const char2 *>(chan_in), static_cast<int2 *>(h.acc), h.n_in,
+                                               h.n_spectra, h.n_base, n_blk, n_split, store ? 1 : 0);
+        } else {
+            auto kern = (h.n_spectra % 2) == 0 ? k_xeng_f32_small<true> : k_xeng_f32_small<false>;
+            kern<<<h.n_chan, threads, 0, st>>>(X, static_cast<float2 *>(h.acc), gains, h.n_in, h.n_spectra, h.n_base,
+                                               n_blk, n_split, store ? 1 : 0);
+        }
+    } else if (h.precision == CORR_PREC_INT8) {
         const int nb = (h.n_in + TB - 1) / TB;
         dim3 grid(nb * (nb + 1) / 2, h.n_chan);
         k_xeng_i8<<<grid, NTH, 0, st>>>(static_cast<const char2 *>(chan_in), static_cast<int2 *>(h.acc), h.n_in,
                                         h.n_spectra, h.n_base, store ? 1 : 0);
-    } else if (h.n_in <= kSmallIn) {
-        const int nb = (h.n_in + 3) / 4, n_blk = nb * (nb + 1) / 2;
-        // K ranges: as many warps as fit in 20, as long as each range has a few rounds
-        const int n_split = std::max(1, std::min(20 / n_blk, h.n_spectra / 256));
-        auto kern = (h.n_spectra % 2) == 0 ? k_xeng_f32_small<true> : k_xeng_f32_small<false>;
-        kern<<<h.n_chan, 32 * n_blk * n_split, 0, st>>>(X, static_cast<float2 *>(h.acc), gains, h.n_in, h.n_spectra,
-                                                        h.n_base, n_blk, n_split, store ? 1 : 0);
     } else {
         const int ct = f32_tile_ct(h);
         s = ct == 2 ? launch_f32<2>(h, X, gains, store, st)
