@@ -163,8 +163,8 @@ corr_status launch_adj(const Handle &h, const float2 *G, const float2 *X, const 
     const int nM = (h.n_in + C::TM - 1) / C::TM, nA = (h.n_spectra + TA - 1) / TA;
     const long long n = (long long)nM * nA * h.n_chan;
     if (n > 0x7fffffffLL) return CORR_EUNSUPPORTED;
-    auto kern = k_adj<RT>;
-    CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
+    constexpr auto kern = k_adj<RT>;
+    if (const corr_status e = allow_smem<kern>((int)C::smem); e != CORR_OK) return e;
     kern<<<(unsigned)n, kFtNth, C::smem, st>>>(G, X, gains, dX, part, h.n_in, h.n_spectra, h.n_base, nM, nA);
     return check_launch("k_adj");
 }

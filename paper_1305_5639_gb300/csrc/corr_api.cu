@@ -262,8 +262,15 @@ static corr_status fx_host_run(corr_t *c, const void *volt_host, const float *ch
         const corr_status s = corr::flush_dump(h, st);  // this pipeline dumps per channel block itself
         if (s != CORR_OK) return s;
     }
-    constexpr int NB = 8, NC = 8;  // input blocks (copy-in || F-engine), channel blocks (X + dump || copy-out)
+    // input blocks (copy-in || F-engine) and channel blocks (X + dump || copy-out): up to 8,
+    // of 2 MB at least, below which a block's copy is shorter than the calls that issue it
+    // (7 inputs x 80 spectra at N = 4096, 4.6 MB in: 396 -> 189 us)
+    constexpr int NB = 8, NC = 8;
+    constexpr size_t kMinBlock = (size_t)2 << 20;
     const size_t volt_bytes = (size_t)h.n_in * h.n_spectra * h.n_chan * 2;
+    const size_t out_bytes = (size_t)h.n_chan * h.n_base * (accum_out ? sizeof(int2) : sizeof(double2));
+    const int nb = (int)std::min<size_t>(NB, std::max<size_t>(1, volt_bytes / kMinBlock));
+    const int nc = (int)std::min<size_t>(NC, std::max<size_t>(1, out_bytes / kMinBlock));
     const size_t chan_bytes = (size_t)h.n_chan * 2 * h.n_in * h.n_spectra * 2;
     if (!h.fx_ready) {
         // all or nothing: a failed allocation or creation releases whatever this
@@ -293,8 +300,8 @@ static corr_status fx_host_run(corr_t *c, const void *volt_host, const float *ch
     void *const vdev = h.fx_volt[par];
     CORR_CUDA_TRY(cudaStreamWaitEvent(h.fx_in, ev[NB + NC + 2 + par], 0));
     const size_t row = (size_t)h.n_spectra * h.n_chan * 2;  // bytes of one input's time series
-    const int ib = (h.n_in + NB - 1) / NB;
-    for (int b = 0; b < NB; ++b) {
+    const int ib = (h.n_in + nb - 1) / nb;
+    for (int b = 0; b < nb; ++b) {
         const int i0 = b * ib, i1 = std::min(h.n_in, i0 + ib);
         if (i1 > i0) {
             CORR_CUDA_TRY(cudaMemcpyAsync(static_cast<char *>(vdev) + row * i0,
@@ -310,8 +317,8 @@ static corr_status fx_host_run(corr_t *c, const void *volt_host, const float *ch
     CORR_CUDA_TRY(cudaEventRecord(ev[NB + NC + 2 + par], st));
     const bool fused = (h.flags & CORR_FLAG_FUSED_DUMP) != 0;
     const bool store = h.acc_zero;
-    const int cb = (h.n_chan + NC - 1) / NC;
-    for (int k = 0; k < NC; ++k) {
+    const int cb = (h.n_chan + nc - 1) / nc;
+    for (int k = 0; k < nc; ++k) {
         const int c0 = k * cb, c1 = std::min(h.n_chan, c0 + cb);
         corr_status s = corr::launch_xengine_tma_range(h, h.fx_chan, 2, nullptr, nullptr, h.n_spectra, store, c0, c1,
                                                        st);

@@ -719,8 +719,8 @@ template <int N, bool I8, int MODE, int FEAT, int P = 0>
 corr_status launch_one_(const FShape &f, const void *volt, const float *scale, void *out, double *power,
                        cudaStream_t st, const PfbArgs &pfb = {}) {
     using C = FCfg<N, I8, MODE, FEAT>;
-    auto kern = k_fengine<N, I8, MODE, FEAT, P>;
-    CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
+    constexpr auto kern = k_fengine<N, I8, MODE, FEAT, P>;
+    if (const corr_status s = allow_smem<kern>((int)C::smem); s != CORR_OK) return s;
     // 16-byte row stores need 16-byte aligned rows: an aligned buffer and 8 | n_spectra
     const int vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0) && (f.n_spectra % 8 == 0);
     // blockIdx.x (the spectra block) varies fastest, so the CTAs resident at one time

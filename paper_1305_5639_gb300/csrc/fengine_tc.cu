@@ -509,10 +509,10 @@ corr_status launch_fengine_tc(const Handle &h, const void *volt, const float *sc
     if (n_items >= (1ll << 28)) return CORR_EINVAL;  // 32-bit item arithmetic in the kernel
     const unsigned grid = (unsigned)(n_items < h.n_sm ? n_items : h.n_sm);
     if (h.flags & CORR_FLAG_PLANAR) {
-        CORR_CUDA_TRY(cudaFuncSetAttribute(k_fengine_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+        if (const corr_status s = allow_smem<k_fengine_tc<true>>(kSmemBytes); s != CORR_OK) return s;
         k_fengine_tc<true><<<grid, kFtThreads, kSmemBytes, st>>>(p);
     } else {
-        CORR_CUDA_TRY(cudaFuncSetAttribute(k_fengine_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes));
+        if (const corr_status s = allow_smem<k_fengine_tc<false>>(kSmemBytes); s != CORR_OK) return s;
         k_fengine_tc<false><<<grid, kFtThreads, kSmemBytes, st>>>(p);
     }
     return check_launch("k_fengine_tc");

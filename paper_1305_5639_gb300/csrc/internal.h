@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 #include "corr.h"
@@ -103,20 +104,38 @@ corr_status check_launch(const char *what);
         }                                                    \
     } while (0)
 
-// Makes a device current for the lifetime of the guard and restores the previous one.
+// Makes a device current for the lifetime of the guard and restores the previous one
+// (nothing to do at either end where it is current already).
 struct DeviceGuard {
     int prev = -1;
-    bool ok = true;
+    bool ok = true, changed = false;
     explicit DeviceGuard(int dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        if (dev >= 0 && dev != prev) ok = cudaSetDevice(dev) == cudaSuccess;
+        if (dev >= 0 && dev != prev) {
+            ok = cudaSetDevice(dev) == cudaSuccess;
+            changed = true;
+        }
     }
     ~DeviceGuard() {
-        if (prev >= 0) cudaSetDevice(prev);
+        if (changed && prev >= 0) cudaSetDevice(prev);
     }
     DeviceGuard(const DeviceGuard &) = delete;
     DeviceGuard &operator=(const DeviceGuard &) = delete;
 };
+
+// Raises the dynamic shared memory limit of kernel Kern on the current device to `bytes`,
+// once per device (the attribute stays; it was set before every launch, 0.5 us each).
+template <auto Kern>
+corr_status allow_smem(int bytes) {
+    static std::atomic<unsigned long long> done{0};  // devices 0 .. 63
+    int dev = -1;
+    CORR_CUDA_TRY(cudaGetDevice(&dev));
+    const unsigned long long bit = dev >= 0 && dev < 64 ? 1ull << dev : 0ull;
+    if (bit && (done.load(std::memory_order_acquire) & bit)) return CORR_OK;
+    CORR_CUDA_TRY(cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    done.fetch_or(bit, std::memory_order_release);
+    return CORR_OK;
+}
 
 // Kernel launchers (return CORR_OK or an error status).
 corr_status launch_fengine(const Handle &h, const void *volt, const float *scale, void *out,

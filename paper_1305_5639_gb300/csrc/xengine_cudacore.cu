@@ -127,8 +127,8 @@ corr_status launch_f32(const Handle &h, const float2 *X, const float2 *gains, bo
     const int nb = (h.n_in + C::TB - 1) / C::TB;
     const long long n_tiles = (long long)nb * (nb + 1) / 2;
     if (n_tiles * h.n_chan > 0x7fffffffLL) return CORR_EUNSUPPORTED;
-    auto kern = k_xeng_f32<CT>;
-    CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem));
+    constexpr auto kern = k_xeng_f32<CT>;
+    if (const corr_status e = allow_smem<kern>((int)C::smem); e != CORR_OK) return e;
     kern<<<(unsigned)(n_tiles * h.n_chan), kFtNth, C::smem, st>>>(X, static_cast<float2 *>(h.acc), gains, h.n_in,
                                                                  h.n_spectra, h.n_base, (int)n_tiles, store ? 1 : 0);
     return CORR_OK;

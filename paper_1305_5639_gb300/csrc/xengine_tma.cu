@@ -972,8 +972,8 @@ corr_status tma_encode_planar(void *tmap128, const void *planes, int n_in, int n
 // Every INT8 launch but the short-time one: the wide form, 640 threads.
 corr_status launch_int8_wide(const CUtensorMap &tmap, const TParams &p, unsigned grid, cudaStream_t st) {
     using C = TCfg<2, 64>;
-    auto kern = k_xeng_tma<kInt8, C, false, true>;
-    CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
+    constexpr auto kern = k_xeng_tma<kInt8, C, false, true>;
+    if (const corr_status e = allow_smem<kern>(C::SMEM_BYTES); e != CORR_OK) return e;
     kern<<<grid, NTHREADS_WIDE, C::SMEM_BYTES, st>>>(tmap, tmap, p);
     return CORR_OK;
 }
@@ -982,13 +982,13 @@ corr_status launch_int8_wide(const CUtensorMap &tmap, const TParams &p, unsigned
 corr_status launch_fp16_wide(const CUtensorMap &tmap, const TParams &p, int npl, unsigned grid, cudaStream_t st) {
     if (npl == 2) {
         using C = TCfg<2, 64>;
-        auto kern = k_xeng_tma<kFp16, C, false, true>;
-        CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
+        constexpr auto kern = k_xeng_tma<kFp16, C, false, true>;
+        if (const corr_status e = allow_smem<kern>(C::SMEM_BYTES); e != CORR_OK) return e;
         kern<<<grid, NTHREADS_WIDE, C::SMEM_BYTES, st>>>(tmap, tmap, p);
     } else {
         using C = TCfg<4, 32>;
-        auto kern = k_xeng_tma<kFp16, C, false, true>;
-        CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
+        constexpr auto kern = k_xeng_tma<kFp16, C, false, true>;
+        if (const corr_status e = allow_smem<kern>(C::SMEM_BYTES); e != CORR_OK) return e;
         kern<<<grid, NTHREADS_WIDE, C::SMEM_BYTES, st>>>(tmap, tmap, p);
     }
     return CORR_OK;
@@ -1070,8 +1070,8 @@ corr_status launch_xengine_tma_range(const Handle &h, const void *planes, int np
     StageScope sc(h, CORR_STAGE_XENGINE, st);
     if (h.precision == CORR_PREC_INT8 && p.st_out) {
         using C = TCfg<2, 64>;
-        auto kern = k_xeng_tma<kInt8, C, true>;
-        CORR_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
+        constexpr auto kern = k_xeng_tma<kInt8, C, true>;
+        if (const corr_status e = allow_smem<kern>(C::SMEM_BYTES); e != CORR_OK) return e;
         kern<<<grid, NTHREADS_WIDE, C::SMEM_BYTES, st>>>(tmap, tmap, p);
     } else if (h.precision == CORR_PREC_INT8) {
         const corr_status s = launch_int8_wide(tmap, p, grid, st);
@@ -1192,7 +1192,7 @@ corr_status launch_adjoint_tma(const Handle &h, const void *a_planes, const void
     p.expo = expo;
     const unsigned grid = (unsigned)(p.n_items < h.n_sm ? p.n_items : h.n_sm);
     StageScope sc(h, CORR_STAGE_ADJ_GEMM, st);
-    CORR_CUDA_TRY(cudaFuncSetAttribute(k_xeng_tma<kAdj, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES));
+    if ((s = allow_smem<k_xeng_tma<kAdj, C>>(C::SMEM_BYTES)) != CORR_OK) return s;
     k_xeng_tma<kAdj, C><<<grid, NTHREADS, C::SMEM_BYTES, st>>>(ta, tb, p);
     return check_launch("k_xeng_tma (adjoint)");
 }
