@@ -157,13 +157,15 @@ int f32_tile_ct(const Handle &h) {
 // sums of a block (16 pairs, Re and Im) are then added over the lanes by a transposing
 // butterfly that leaves sum number `lane` in each lane, and over the K ranges in order: a
 // fixed order, so the result is run-to-run identical. Bound by the L1 reads (each row is
-// read by the n_in / 4 + 1 blocks it meets) and the FP32 pipe: 14.5 us for 16 inputs, 256
+// read by the n_in / 4 + 1 blocks it meets) and the FP32 pipe: 14 us for 16 inputs, 256
 // channels, 1024 spectra (33.5 MB: 5 us of HBM time), against 30.4 us with one thread per
-// pair reading both factors of each product from shared memory. Above 32 inputs the tiles
+// pair reading both factors of each product from shared memory. Twelve warps, two CTAs per
+// SM: three tasks each at 36 blocks, and one CTA's reduction beside the other's loads (16
+// inputs: 18.5 us with the dump against 20.8 with 20 warps, one CTA). Above 32 inputs the tiles
 // of k_xeng_f32 have the better ratio of sums to reads (24 inputs, 256 channels, 1024
 // spectra: 35 us here, 60 us there).
 constexpr int kSmallIn = 32;     // at most 36 blocks
-constexpr int kSmallWarps = 20;
+constexpr int kSmallWarps = 12;
 constexpr int kSmallTasks = 36;  // blocks x K ranges
 
 // the sums v[k] of all lanes: afterwards v[0] holds sum number `lane`
@@ -184,7 +186,7 @@ __device__ __forceinline__ void butterfly32(T (&v)[32], int lane) {
 }
 
 template <bool VEC>
-__global__ void __launch_bounds__(32 * kSmallWarps) k_xeng_f32_small(const float2 *__restrict__ X, float2 *__restrict__ acc,
+__global__ void __launch_bounds__(32 * kSmallWarps, 2) k_xeng_f32_small(const float2 *__restrict__ X, float2 *__restrict__ acc,
                                                          const float2 *__restrict__ gains, int n_in, int K,
                                                          long long B, int n_blk, int n_split, int store) {
     __shared__ float part[kSmallTasks][32];
@@ -274,10 +276,10 @@ constexpr int kImOnes = 0x01000100;
 // single spectra), every word feeding four dp4a pairs. Reads the complex int8 layout
 // directly, where the tensor cores need a conversion pass and spend a 128 x 128 tile on the
 // few pairs. X-engine and dump, tensor cores -> here (us): 16 inputs, 256 channels, 1024
-// spectra 39 -> 15; 8 inputs, 1024 channels, 512 spectra 70 -> 15; 32 inputs, 1024 channels,
-// 4096 spectra 471 -> 245.
+// spectra 39 -> 13; 8 inputs, 1024 channels, 512 spectra 70 -> 12; 32 inputs, 1024 channels,
+// 4096 spectra 471 -> 233.
 template <int W>
-__global__ void __launch_bounds__(32 * kSmallWarps) k_xeng_i8_small(const char2 *__restrict__ X, int2 *__restrict__ acc,
+__global__ void __launch_bounds__(32 * kSmallWarps, 2) k_xeng_i8_small(const char2 *__restrict__ X, int2 *__restrict__ acc,
                                                                     int n_in, int K, long long B, int n_blk,
                                                                     int n_split, int store) {
     __shared__ int part[kSmallTasks][32];
