@@ -250,23 +250,26 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fengine_tc(const FtParams p) 
             for (int gs = 0; gs < 4 && alive; ++gs) alive = issue(gs);
         alive = __shfl_sync(0xffffffffu, alive ? 1 : 0, 0) != 0;
         int i = 0, a0 = 0;  // the current item
+        // lanes 0-15 take frame 2 cw, lanes 16-31 frame 2 cw + 1; lane u = lane % 16 owns
+        // rows t = 2u, 2u + 1, whose samples share one 32-bit word of each raw row m
+        const int q = 2 * cw + (lane >> 4), u = lane & 15;
+        // tile rows of t = 2u and t = 2u + 1: 32 q + u and 32 q + 16 + u (2048 bytes on); the
+        // 16-byte chunk kc of row r lies at chunk kc ^ (r % 8)
+        uint32_t arow[8];
+#pragma unroll
+        for (int kc = 0; kc < 8; ++kc) arow[kc] = sbase + OFF_A1 + sw128_off(32 * q + u, 8 * kc);
         for (int gs = 0; gs < total && alive; ++gs) {
             const int b = gs & 1, s = gs & 3;
             const uint32_t ph = (uint32_t)((gs >> 1) & 1);
             if (!wwait(B_RF + s, (uint32_t)((gs >> 2) & 1)) || !wwait(B_A1E + b, ph ^ 1u)) break;
             if (s == 0) item_of(gs >> 2, i, a0);
-            // lanes 0-15 take frame 2 cw, lanes 16-31 frame 2 cw + 1; lane u = lane % 16 owns
-            // rows t = 2u, 2u + 1, whose samples share one 32-bit word of each raw row m
-            const uint32_t atile = sbase + OFF_A1 + b * kTileA;
-            const int q = 2 * cw + (lane >> 4), u = lane & 15;
             const bool valid = a0 + 4 * (gs & 3) + q < p.K;
             const uint32_t rs = sbase + OFF_RAW + s * kRawSlot + q * 2 * kFtN + 4 * u;
             uint32_t w[kFtR];
 #pragma unroll
             for (int m = 0; m < kFtR; ++m) w[m] = valid ? lds_u32(rs + 2 * kFtR * m) : 0u;
-            // rows of t = 2u and t = 2u + 1 (tile rows 32 q + u and 32 q + 16 + u): columns
-            // (m, Re / Im), 16-byte chunks of 4 m
-            const int r0 = 32 * q + u;
+            // columns (m, Re / Im), 16-byte chunks of 4 m
+            const uint32_t tile = (uint32_t)b * kTileA;
 #pragma unroll
             for (int kc = 0; kc < 8; ++kc) {
                 uint4 va, vb;
@@ -274,8 +277,8 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fengine_tc(const FtParams p) 
                 i8x2_to_h2(w[4 * kc + 1], va.y, vb.y);
                 i8x2_to_h2(w[4 * kc + 2], va.z, vb.z);
                 i8x2_to_h2(w[4 * kc + 3], va.w, vb.w);
-                sts_v4(atile + sw128_off(r0, 8 * kc), va);
-                sts_v4(atile + sw128_off(r0 + 16, 8 * kc), vb);
+                sts_v4(arow[kc] + tile, va);
+                sts_v4(arow[kc] + tile + 2048, vb);
             }
             tc::fence_proxy_async_smem();
             __syncwarp();
@@ -300,25 +303,35 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fengine_tc(const FtParams p) 
             if (nv == kFtSB && p.vec_out) {
                 // each lane moves 8 spectra of one channel row: 4 staged words -> one
                 // 16-byte store per plane; 16 rows per pass
+                // (row k = 16 it + lane / 2: its word swizzle (k / 4) % 8 depends on it's parity)
                 const int c8 = lane & 1;
-                const size_t dplane = (size_t)p.n_in * p.K / 8;
-#pragma unroll 4
-                for (int k = lane >> 1; k < kFtN; k += 16) {
-                    const int h = (k >> kFtSw) & (kFtRoww - 1);
-                    const uint32_t src = stg_s + 4u * (uint32_t)(k * kFtRoww);
-                    const uint32_t w0 = lds_u32(src + 4 * ((4 * c8) ^ h)), w1 = lds_u32(src + 4 * ((4 * c8 + 1) ^ h));
-                    const uint32_t w2 = lds_u32(src + 4 * ((4 * c8 + 2) ^ h)), w3 = lds_u32(src + 4 * ((4 * c8 + 3) ^ h));
-                    uint4 *d = reinterpret_cast<uint4 *>(dst + ((size_t)(PL * k) * p.n_in + i) * p.K + a0 + 8 * c8);
-                    if constexpr (PLANAR) {
-                        uint4 re, im;
-                        ob_codes_to_f16_planes(w0, re.x, im.x);
-                        ob_codes_to_f16_planes(w1, re.y, im.y);
-                        ob_codes_to_f16_planes(w2, re.z, im.z);
-                        ob_codes_to_f16_planes(w3, re.w, im.w);
-                        d[0] = re;
-                        d[dplane] = im;
-                    } else {
-                        d[0] = make_uint4(w0, w1, w2, w3);
+                const size_t dplane = (size_t)p.n_in * p.K / 8, dstep = 16 * PL * dplane;
+                uint4 *d = reinterpret_cast<uint4 *>(dst + ((size_t)(PL * (lane >> 1)) * p.n_in + i) * p.K + a0 + 8 * c8);
+                uint32_t src[2][4];
+#pragma unroll
+                for (int par = 0; par < 2; ++par) {
+                    const int k = 16 * par + (lane >> 1), h = (k >> kFtSw) & (kFtRoww - 1);
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) src[par][x] = stg_s + 4u * (uint32_t)(k * kFtRoww + ((4 * c8 + x) ^ h));
+                }
+#pragma unroll 2
+                for (int it = 0; it < kFtN / 16; it += 2) {
+#pragma unroll
+                    for (int par = 0; par < 2; ++par, d += dstep) {
+                        const uint32_t o = (uint32_t)(it * 16 * kFtRoww * 4);
+                        const uint32_t w0 = lds_u32(src[par][0] + o), w1 = lds_u32(src[par][1] + o);
+                        const uint32_t w2 = lds_u32(src[par][2] + o), w3 = lds_u32(src[par][3] + o);
+                        if constexpr (PLANAR) {
+                            uint4 re, im;
+                            ob_codes_to_f16_planes(w0, re.x, im.x);
+                            ob_codes_to_f16_planes(w1, re.y, im.y);
+                            ob_codes_to_f16_planes(w2, re.z, im.z);
+                            ob_codes_to_f16_planes(w3, re.w, im.w);
+                            d[0] = re;
+                            d[dplane] = im;
+                        } else {
+                            d[0] = make_uint4(w0, w1, w2, w3);
+                        }
                     }
                 }
             } else {
@@ -360,6 +373,11 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fengine_tc(const FtParams p) 
         float2 tw[16];                               // W_1024^(t k1)
 #pragma unroll
         for (int j = 0; j < 16; ++j) tw[j] = __ldg(p.tw + (16 * kh + j) * kFtR + t);
+        // byte offset of element (row 32 q + 16 kh + j, column pair t) for j < 8; j + 8 lies
+        // 1024 bytes on
+        uint32_t a2row[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) a2row[j] = sbase + OFF_A2H + sw128_off(32 * q + 16 * kh + j, 2 * t);
         for (int gs = 0; gs < total; ++gs) {
             const int b = gs & 1, c = gs & 3;
             const uint32_t ph = (uint32_t)((gs >> 1) & 1);
@@ -376,21 +394,21 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fengine_tc(const FtParams p) 
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 float2 y = make_float2(__uint_as_float(yh[2 * j]), __uint_as_float(yh[2 * j + 1]));
-                if (kh != 0 || j != 0) y = cmul(y, tw[j]);
+                if (kh != 0 || j != 0) y = cmul2(y, tw[j]);
                 const __half2 h = __floats2half2_rn(y.x, y.y);
-                const float2 hf = __half22float2(h);
-                const __half2 l = __floats2half2_rn(y.x - hf.x, y.y - hf.y);
+                const float2 r = f2_sub(y, __half22float2(h));
+                const __half2 l = __floats2half2_rn(r.x, r.y);
                 yh[2 * j] = *reinterpret_cast<const uint32_t *>(&h);
                 yh[2 * j + 1] = *reinterpret_cast<const uint32_t *>(&l);
             }
             if (!wwait(B_A2E + b, ph ^ 1u)) break;
-            const uint32_t ah = sbase + OFF_A2H + b * kTileA, al = sbase + OFF_A2L + b * kTileA;
+            const uint32_t tile = (uint32_t)b * kTileA;
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 // row (q, k1) of stage 2's A tiles, column pair (t, Re / Im)
-                const uint32_t off = sw128_off(32 * q + 16 * kh + j, 2 * t);
-                sts_u32(ah + off, yh[2 * j]);
-                sts_u32(al + off, yh[2 * j + 1]);
+                const uint32_t at = a2row[j & 7] + tile + (j & 8) * 128;
+                sts_u32(at, yh[2 * j]);
+                sts_u32(at + (OFF_A2L - OFF_A2H), yh[2 * j + 1]);
             }
             tc::fence_proxy_async_smem();
             __syncwarp();
@@ -412,7 +430,9 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fengine_tc(const FtParams p) 
             if (!wwait(B_D2F + c, (uint32_t)((gs >> 2) & 1))) break;
             tc::tc_fence_after();
             const int s = 4 * g + q;  // spectrum within the item
-            const uint32_t stg_s = sbase + OFF_STG + (int)(r & 1) * kStgBytes;
+            // slot of code (lane, s); channel lane + 32 k2 has the same swizzle, 32 rows on
+            const uint32_t slot0 = sbase + OFF_STG + (uint32_t)(r & 1) * kStgBytes + 2u * (uint32_t)stg_slot(lane, s);
+            constexpr uint32_t kRow32 = kFtR * kFtRoww * 4;
             // X, 16 k2 at a time
 #pragma unroll
             for (int hlf = 0; hlf < 2; ++hlf) {
@@ -432,7 +452,7 @@ __global__ void __launch_bounds__(kFtThreads, 1) k_fengine_tc(const FtParams p) 
                         xa[j] = pack_q<PLANAR>(x, sc[k2]);
                     }
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) sts_u16(stg_s + 2 * stg_slot(lane + kFtR * (16 * hlf + j), s), xa[j]);
+                    for (int j = 0; j < 16; ++j) sts_u16(slot0 + (16 * hlf + j) * kRow32, xa[j]);
                 }
             }
             if (g == 3) {
