@@ -269,7 +269,7 @@ __device__ __forceinline__ void pfb_frames(float *slots, const char2 *__restrict
 // int8 layout (us): N = 2048 x 1024 spectra 555 -> 324 (the T2-point DFTs ran on one of two
 // warps, at 212 registers and 8 warps per SM), N = 4096 x 512 527 -> 445 (8 -> 16 warps), N =
 // 512 x 4096 346 -> 258 and N = 128 x 16384 338 -> 267 (half of each warp idle).
-template <int L, int HB>
+template <int L, int HB, bool PACK>
 __device__ __forceinline__ void dft_shared(const float2 (&lo)[L / 4], const float2 (&hi)[L / 4], int h,
                                            float2 (&v)[L / 2]) {
     constexpr int q = L / 4;
@@ -290,9 +290,9 @@ __device__ __forceinline__ void dft_shared(const float2 (&lo)[L / 4], const floa
         const float2 keep = h ? d : s, give = h ? s : d;
         const float2 got = make_float2(__shfl_xor_sync(0xffffffffu, give.x, HB), __shfl_xor_sync(0xffffffffu, give.y, HB));
         v[i] = f2_add(keep, got);
-        v[i + q] = mul_w<i, L / 2>(f2_mul(f2_sub(keep, got), sgn));
+        v[i + q] = mul_w<i, L / 2, PACK>(f2_mul(f2_sub(keep, got), sgn));
     });
-    fft_dif<L / 2, L / 2, 1>(v);
+    fft_dif<L / 2, L / 2, 1, PACK>(v);
 }
 
 template <int N, bool I8, int MODE, int FEAT, int P = 0>
@@ -310,6 +310,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
     constexpr int NT = C::NT, H1 = C::H1, H2 = C::H2;
     constexpr int R1 = T1 / H1, R2 = T2 / H2;  // values per thread in each pass
     constexpr int TV = R1 > R2 ? R1 : R2;
+    constexpr bool PACK = N == 512 || N == 1024 || (N == 4096 && FEAT != kDelay);  // packed factors pay (see mul_w)
     constexpr int HB = T1 < 16 ? T1 : 16;      // lane bit between two threads that share a DFT
     // square 32-point passes read the exchange into float arrays and do pass 2's
     // first stage in scalar arithmetic (no register moves into the (re, im) pairs); the
@@ -486,12 +487,12 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
         }
         // v[bitrev(k')] = Y[col][k1], k1 = H1 k' + h1 (x 256, bin 0 offset, for int8 input)
         if constexpr (H1 == 1) {
-            fft_dif<T1>(v);
+            fft_dif<T1, TV, 0, PACK>(v);
         } else {
             float2 lo[R1 / 2], hi[R1 / 2];
 #pragma unroll
             for (int m = 0; m < R1 / 2; ++m) lo[m] = v[m], hi[m] = v[m + R1 / 2];
-            dft_shared<T1, HB>(lo, hi, h1, v);
+            dft_shared<T1, HB, PACK>(lo, hi, h1, v);
         }
         if constexpr (SCALED) v[0] = h1 == 0 ? kOffsetFix<T1>(v[0]) : v[0];
         sfor<0, R1>([&](auto K1) {
@@ -536,7 +537,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
             }
             group_sync();
             if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
-            dft_shared<T2, HB>(lo, hi, h2, v);  // v[bitrev(k')] = X[row + T1 k2], k2 = 2 k' + h2
+            dft_shared<T2, HB, PACK>(lo, hi, h2, v);  // v[bitrev(k')] = X[row + T1 k2], k2 = 2 k' + h2
         } else if constexpr (kScalarStage) {
             // the rows are read into plain float arrays (a 16-byte load fills four
             // consecutive registers, which the (re, im) register pairs of v cannot offer)
@@ -572,9 +573,9 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
                 if constexpr (4 * a == T2)
                     v[b] = make_float2(ai - bi, br - ar);  // (x - y)(-j)
                 else
-                    v[b] = mul_w<a, T2>(make_float2(ar - br, ai - bi));
+                    v[b] = mul_w<a, T2, PACK>(make_float2(ar - br, ai - bi));
             });
-            fft_dif<T2, TV, 1>(v);  // v[bitrev(k2)] = X[t + T1 k2]
+            fft_dif<T2, TV, 1, PACK>(v);  // v[bitrev(k2)] = X[t + T1 k2]
         } else {
             {
 #pragma unroll
@@ -598,7 +599,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg
             }
             group_sync();
             if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
-            fft_dif<T2>(v);  // v[bitrev(k2)] = X[t + T1 k2]
+            fft_dif<T2, TV, 0, PACK>(v);  // v[bitrev(k2)] = X[t + T1 k2]
         }
         if (PFB && has_dly) {
             // delay phases exp(+j 2 pi T1 k2 f / N), in a block of their own: without delays
