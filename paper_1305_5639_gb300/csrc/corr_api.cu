@@ -184,10 +184,11 @@ void note_capture(Handle &h, cudaStream_t st) {
 }
 
 // Complete a deferred dump now (the dump kernel on the pending accumulator).
-corr_status flush_dump(Handle &h, cudaStream_t st) {
+// out, if not null, also receives the long integration.
+corr_status flush_dump(Handle &h, cudaStream_t st, double2 *out = nullptr) {
     if (!h.dump_pending) return CORR_OK;
     h.vis_zero = false;
-    const corr_status s = launch_dump_src(h, h.pending_src, st);
+    const corr_status s = launch_dump_src(h, h.pending_src, out, st);
     if (s == CORR_OK) h.dump_pending = false;
     return s;
 }
@@ -694,6 +695,9 @@ corr_status corr_dump(corr_t *c, double *vis_out, void *stream) {
     corr::DeviceGuard dg(h.device);
     cudaStream_t st = corr::as_stream(stream);
     corr::note_capture(h, st);
+    // the dump writes the copy along with the sums, where its 16-byte stores are aligned
+    double2 *out = corr::aligned16(vis_out) ? reinterpret_cast<double2 *>(vis_out) : nullptr;
+    bool copied = false;
     if (!h.acc_zero && !(h.flags & CORR_FLAG_FUSED_DUMP)) {
         corr_status s = CORR_OK;
         bool deferred = false;
@@ -714,17 +718,20 @@ corr_status corr_dump(corr_t *c, double *vis_out, void *stream) {
         if (!deferred) {
             h.vis_zero = false;
             s = corr::flush_dump(h, st);
-            if (s == CORR_OK) s = corr::launch_dump(h, st);
+            if (s == CORR_OK) s = corr::launch_dump_src(h, h.acc, out, st);
+            copied = out != nullptr;
         }
         if (s != CORR_OK) return s;
     }
     h.acc_zero = true;
     h.acc_spectra = 0;
-    if (vis_out) {
-        corr_status s = corr::flush_dump(h, st);
+    if (vis_out && !copied) {
+        copied = h.dump_pending && out;
+        corr_status s = corr::flush_dump(h, st, out);
         if (s != CORR_OK) return s;
-        CORR_CUDA_TRY(cudaMemcpyAsync(vis_out, h.vis64, (size_t)h.n_chan * h.n_base * sizeof(double2),
-                                      cudaMemcpyDeviceToDevice, st));
+        if (!copied)
+            CORR_CUDA_TRY(cudaMemcpyAsync(vis_out, h.vis64, (size_t)h.n_chan * h.n_base * sizeof(double2),
+                                          cudaMemcpyDeviceToDevice, st));
     }
     return CORR_OK;
 }

@@ -145,10 +145,10 @@ corr_status launch_xengine_cudacore(const Handle &h, const void *chan_in, const 
                                     bool store, cudaStream_t st);
 // Whether an AUTO INT8 X-engine call runs on the CUDA cores: complex int8 layout, few inputs.
 bool xengine_i8_small(const Handle &h);
-corr_status launch_dump(const Handle &h, cudaStream_t st);
 corr_status launch_dump_range(const Handle &h, int c0, int c1, cudaStream_t st);
-// The dump of an accumulator other than the handle's current one (a deferred dump).
-corr_status launch_dump_src(const Handle &h, const void *acc, cudaStream_t st);
+// The dump of a whole accumulator (the handle's current one, or a deferred dump's); out, if
+// not null, also receives the long integration.
+corr_status launch_dump_src(const Handle &h, const void *acc, double2 *out, cudaStream_t st);
 corr_status launch_fengine_range(const Handle &h, const void *volt, const float *scale, void *out, int i0, int n_run,
                                  cudaStream_t st);
 // TMA X-engine over channels [c0, c1) of planar FP16 operands [chan][npl][n_in][kstride]
