@@ -438,7 +438,7 @@ corr_status corr_create(int32_t n_ant, int32_t n_pol, int32_t n_chan, int32_t n_
     const size_t nvis = (size_t)h.n_chan * (size_t)h.n_base;
     const size_t acc_bytes = nvis * 8;  // int2 or float2
     bool ok = cudaMalloc(&h.acc, acc_bytes) == cudaSuccess && cudaMalloc(&h.vis64, nvis * sizeof(double2)) == cudaSuccess &&
-              cudaMalloc(&h.status, sizeof(int32_t)) == cudaSuccess &&
+              cudaMalloc(&h.status, 3 * sizeof(int32_t)) == cudaSuccess &&
               cudaMalloc(&h.power64, sizeof(double) * (size_t)n_chan) == cudaSuccess;
     if (ok && corr::fengine_supported(n_chan)) ok = cudaMalloc(&h.twiddle, sizeof(float2) * (size_t)n_chan) == cudaSuccess;
     if (!ok) {
@@ -448,7 +448,7 @@ corr_status corr_create(int32_t n_ant, int32_t n_pol, int32_t n_chan, int32_t n_
         return CORR_ENOMEM;
     }
     ok = cudaMemset(h.acc, 0, acc_bytes) == cudaSuccess && cudaMemset(h.vis64, 0, nvis * sizeof(double2)) == cudaSuccess &&
-         cudaMemset(h.status, 0, sizeof(int32_t)) == cudaSuccess;
+         cudaMemset(h.status, 0, 3 * sizeof(int32_t)) == cudaSuccess;
     if (ok && h.twiddle) {
         // F-engine twiddles W_N^(t k1) = exp(-j 2 pi t k1 / N) for the N = T1 x T2 split,
         // laid out [k1][t] (k1 < T1, t < T2); computed in double, rounded once to float

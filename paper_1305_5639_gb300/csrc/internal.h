@@ -56,7 +56,8 @@ struct Handle {
     void *pfb_y = nullptr;       //   its FIR output, complex FP32 [n_in][n_spectra][n_chan]
     int32_t *st_out = nullptr;   // short-time visibilities (caller's buffer; null: off)
     int32_t st_block = 0;        //   spectra per block
-    int32_t *status = nullptr;   // device status word (0 ok, else CORR_* code set by a kernel)
+    int32_t *status = nullptr;   // device status word (0 ok, else CORR_* code set by a kernel), then the
+                                 // two counters of the deferred dump (SideDump, xengine_tma.cu)
     double *power64 = nullptr;   // [n_chan] scratch for corr_fengine_power
     void *planar_ws = nullptr;   // FP16 operand planes for the FP16 tensor-core paths (first use)
     size_t planar_ws_bytes = 0;

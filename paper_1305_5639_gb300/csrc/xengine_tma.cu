@@ -123,10 +123,11 @@ struct TParams {
     int *st_out;
     int st_kb, st_nchan;
     // deferred integration dump (see SideDump): side_dst[e] += side_src[e] for e < side_n
-    // (int2 for INT8, float2 for FP16), each CTA a contiguous slice; side_n = 0: none
+    // (int2 for INT8, float2 for FP16); side_n = 0: none
     const void *side_src;
     double2 *side_dst;
     long long side_n;
+    unsigned *side_ctr;  // chunks claimed, CTAs finished (both zero between launches)
 };
 
 // Everything a role needs to know about one work item.
@@ -270,33 +271,29 @@ __device__ __forceinline__ void write_sums16(const int (&R)[64], const Item &itm
 }
 
 // The previous integration's dump into the FP64 long integration, riding along in an
-// X-engine launch. Each CTA owns a contiguous slice, cut into chunks of 256 visibilities
-// that any of its warps claims from a shared counter: warps 2 and 3 (no role in the
-// pipeline) from the start, every other warp once its role has ended. Two warps alone
-// hold too few loads in flight: 38 G visibilities/s, which bound a launch of few spectra
-// (250 inputs, 128 channels, 1504 spectra: 118 -> 91 us with all warps, 76 us without a
-// dump; 128 inputs, 512 channels, 256 spectra: 119 -> 64 us, 37 us without). The
-// sums are exact (integer values below 2^53 for INT8; the FP64 add of the FP32 sums for
-// FP16), as the dump kernel's.
-struct SideState {  // in shared memory, so that the epilogues' registers do not carry it
-    long long lo, hi;         // this CTA's slice
-    unsigned n_chunks, next;  // its chunks, and those claimed so far
-};
-
+// X-engine launch. It is cut into chunks of 256 visibilities that any warp of any CTA claims
+// from a global counter: warps 2 and 3 (no role in the pipeline) from the start, every other
+// warp once its role has ended, so that CTAs with a tile less than others do more of it. Two
+// warps per CTA alone hold too few loads in flight: 38 G visibilities/s, which bound a launch
+// of few spectra (250 inputs, 128 channels, 1504 spectra: 118 us; 91 with all warps and a
+// fixed slice per CTA; 81 with the counter; 68 without a dump; 128 inputs, 512 channels, 256
+// spectra: 119, 64, 59 and 32). The last CTA to finish clears the counters for the next
+// launch. The sums are exact (integer values below 2^53 for INT8; the FP64 add of the FP32
+// sums for FP16), as the dump kernel's.
 template <typename AccT>
 struct SideDump {
     static constexpr int U = 8;             // visibilities per lane and chunk, loads before stores
     static constexpr int kChunk = 32 * U;
-    static constexpr unsigned kAhead = 8;   // chunks prefetched into L2 ahead of the claims
+    static constexpr unsigned kAhead = 2;   // chunks per CTA prefetched into L2 ahead of the claims
     const TParams &p;
-    volatile SideState *st;  // shared
     volatile int *abort_flag;
 
+    __device__ __forceinline__ unsigned n_chunks() const { return (unsigned)((p.side_n + kChunk - 1) / kChunk); }
     // bulk L2 prefetch of chunk c of both streams (one lane; 16-byte aligned ranges
     // inside the buffers)
     __device__ __forceinline__ void prefetch(unsigned c) const {
-        if (c >= st->n_chunks) return;
-        const long long b = st->lo + (long long)c * kChunk, e = min((long long)st->hi, b + kChunk);
+        if (c >= n_chunks()) return;
+        const long long b = (long long)c * kChunk, e = min(p.side_n, b + kChunk);
         const AccT *src = static_cast<const AccT *>(p.side_src);
         const uintptr_t sa = reinterpret_cast<uintptr_t>(src + b) & ~(uintptr_t)15;
         const uintptr_t se = reinterpret_cast<uintptr_t>(src + e) & ~(uintptr_t)15;
@@ -321,13 +318,14 @@ struct SideDump {
     }
     // one chunk by the calling warp (all lanes); false when none is left
     __device__ __forceinline__ bool chunk(int lane) const {
+        const unsigned n = n_chunks();
         unsigned c = 0;
-        if (lane == 0) c = *abort_flag ? st->n_chunks : atomicAdd(const_cast<unsigned *>(&st->next), 1u);
+        if (lane == 0) c = *abort_flag ? n : atomicAdd(p.side_ctr, 1u);
         c = __shfl_sync(0xffffffffu, c, 0);
-        if (c >= st->n_chunks) return false;
-        if (lane == 0) prefetch(c + kAhead);
-        const long long e0 = st->lo + (long long)c * kChunk + lane;
-        add(static_cast<const AccT *>(p.side_src) + e0, p.side_dst + e0, st->hi - e0);
+        if (c >= n) return false;
+        if (lane == 0) prefetch(c + kAhead * gridDim.x);
+        const long long e0 = (long long)c * kChunk + lane;
+        add(static_cast<const AccT *>(p.side_src) + e0, p.side_dst + e0, p.side_n - e0);
         return true;
     }
 };
@@ -399,17 +397,10 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
     const uint32_t drain_bar = bar0 + 8u * (2 * NSTAGE + 4);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(sgen + OFF_BAR + 8 * (2 * NSTAGE + 5));
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
-    SideState *side_st = reinterpret_cast<SideState *>(sgen + OFF_BAR + 128);
     using AccT = typename std::conditional<MODE == kInt8, int2, float2>::type;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        if (p.side_n > 0) {
-            side_st->lo = p.side_n * blockIdx.x / gridDim.x;
-            side_st->hi = p.side_n * (blockIdx.x + 1) / gridDim.x;
-            side_st->n_chunks = (unsigned)((side_st->hi - side_st->lo + SideDump<AccT>::kChunk - 1) / SideDump<AccT>::kChunk);
-            side_st->next = 0;
-        }
         for (int s = 0; s < NSTAGE; ++s) {
             tc::mbar_init(full_bar(s), 1);
             tc::mbar_init(empty_bar(s), 1);
@@ -910,9 +901,7 @@ add_sums<false>(R + 8 * cb, u, w);
 
     if (p.side_n > 0) {
         // deferred dump: warps 2 and 3 from the start, the others when their role has ended
-        const SideDump<AccT> side{p, side_st, abort_flag};
-        if ((warp == 2 || warp == 3) && lane == 0)
-            for (unsigned c = warp - 2; c < SideDump<AccT>::kAhead; c += 2) side.prefetch(c);
+        const SideDump<AccT> side{p, abort_flag};
         while (side.chunk(lane)) {
         }
     }
@@ -921,6 +910,11 @@ add_sums<false>(R + 8 * cb, u, w);
     __syncthreads();
     tc::tc_fence_after();
     if (warp == 1) tc::tmem_dealloc(tmem, 512);
+    // every warp of this CTA has had its last claim refused; after the last CTA's, none is made
+    if (threadIdx.x == 0 && p.side_n > 0 && atomicAdd(p.side_ctr + 1, 1u) == gridDim.x - 1) {
+        p.side_ctr[0] = 0;
+        p.side_ctr[1] = 0;
+    }
 }
 
 // ------------------------------------------------------------------ tensor map
@@ -1050,6 +1044,7 @@ corr_status launch_xengine_tma_range(const Handle &h, const void *planes, int np
         // the previous integration's deferred dump rides along (all channels, one launch)
         p.side_dst = h.vis64;
         p.side_src = h.pending_src;
+        p.side_ctr = reinterpret_cast<unsigned *>(h.status) + 1;
         p.side_n = (long long)h.n_chan * h.n_base;  // (small launches: CTAs without tiles join in)
     }
     p.status = h.status;
