@@ -162,6 +162,24 @@ bool use_tc(const Handle &h) {
     return h.precision != CORR_PREC_FP32;  // FP32 has no tensor-core X-engine
 }
 
+// The FIR output buffer of the two-pass filter bank: one complex FP32 frame per (input,
+// spectrum). Made with the window where the F-engine takes two passes, else by the first
+// power pass (also during a stream capture, which a relaxed capture mode allows).
+corr_status pfb_frames_buffer(Handle &h) {
+    if (h.pfb_y) return CORR_OK;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CORR_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+    const cudaError_t e = cudaMalloc(&h.pfb_y, sizeof(float2) * (size_t)h.n_in * h.n_spectra * h.n_chan);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        h.pfb_y = nullptr;
+        set_error_text("allocating the filter bank's frame buffer failed");
+        return CORR_ENOMEM;
+    }
+    return CORR_OK;
+}
+
 // Integration dumps are deferred into the next X-engine launch, whose warps run them
 // beside the MMAs (see corr_dump and SideDump in xengine_tma.cu): INT8 and FP16 hi/lo on
 // the tensor cores. Plain FP16 dumps at once, so that its calls can be captured and
@@ -554,12 +572,9 @@ corr_status corr_set_pfb(corr_t *c, int32_t n_taps, const float *window) {
     cudaFree(h.pfb_win);
     h.pfb_win = nullptr;
     h.pfb_taps = 0;
-    // the FIR output buffer: one complex FP32 frame per (input, spectrum)
-    const size_t y_bytes = sizeof(float2) * (size_t)h.n_in * h.n_spectra * h.n_chan;
-    if (!h.pfb_y && cudaMalloc(&h.pfb_y, y_bytes) != cudaSuccess) {
-        cudaGetLastError();
-        h.pfb_y = nullptr;
-        return CORR_ENOMEM;
+    if (!corr::pfb_fused(h, n_taps)) {
+        const corr_status s = corr::pfb_frames_buffer(h);
+        if (s != CORR_OK) return s;
     }
     if (cudaMalloc(&h.pfb_win, sizeof(float) * n) != cudaSuccess) {
         cudaGetLastError();
@@ -618,6 +633,10 @@ corr_status corr_fengine_power(corr_t *c, const void *volt, float *power, void *
     if (!corr::fengine_supported(h.n_chan)) return CORR_EUNSUPPORTED;
     if (!corr::aligned16(volt)) return CORR_EINVAL;
     corr::DeviceGuard dg(h.device);
+    if (h.pfb_win) {
+        const corr_status s = corr::pfb_frames_buffer(h);
+        if (s != CORR_OK) return s;
+    }
     return corr::launch_fengine_power(h, volt, power, corr::as_stream(stream));
 }
 

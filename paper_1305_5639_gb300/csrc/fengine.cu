@@ -26,19 +26,10 @@ FShape shape_of(const Handle &h) {
     return f;
 }
 
-// Up to 8 taps on int8 voltages with re-packed output, the filter bank is fused into the
-// F-engine (pfb_frames): the FIR pass wrote 8 bytes per sample and the FFT read them back.
-// 128 inputs x 2 M samples, 4 taps: N = 1024 1361 -> 893 us, N = 256 1101 -> 648, N = 4096
-// 2107 -> 1597; 8 taps at N = 1024 1784 -> 1043. Longer windows (registers per thread), float
-// voltages and the power pass keep the two passes, as does N = 16 (fewer positions than
-// threads).
-bool pfb_fused(const Handle &h) {
-    return h.pfb_win && h.precision == CORR_PREC_INT8 && h.pfb_taps <= 8 && h.n_chan >= 64;
-}
-
-// Otherwise, with the polyphase filter bank the FIR pass forms the tap-weighted frames of inputs
-// [f.i0, f.i0 + n_run) (applying the integer delay advance) into the handle's complex
-// FP32 buffer, and the FFT pass then reads those (float input, phase only).
+// Where the polyphase filter bank is not fused (pfb_fused) the FIR pass forms the
+// tap-weighted frames of inputs [f.i0, f.i0 + n_run) (applying the integer delay advance)
+// into the handle's complex FP32 buffer, and the FFT pass then reads those (float input,
+// phase only).
 corr_status pfb_front(const Handle &h, FShape &f, const void *&volt, cudaStream_t st) {
     if (!h.pfb_win) return CORR_OK;
     StageScope sc(h, CORR_STAGE_PFB, st);
@@ -67,6 +58,14 @@ corr_status power_pass(const FShape &f, const void *volt, double *acc64, float *
 
 }  // namespace
 
+// Up to 8 taps on int8 voltages with re-packed output, the filter bank is fused into the
+// F-engine (pfb_frames): the FIR pass wrote 8 bytes per sample and the FFT read them back.
+// 128 inputs x 2 M samples, 4 taps: N = 1024 1361 -> 893 us, N = 256 1101 -> 648, N = 4096
+// 2107 -> 1597; 8 taps at N = 1024 1784 -> 1043. Longer windows (registers per thread), float
+// voltages and the power pass keep the two passes, as does N = 16 (fewer positions than
+// threads).
+bool pfb_fused(const Handle &h, int taps) { return h.precision == CORR_PREC_INT8 && taps <= 8 && h.n_chan >= 64; }
+
 bool fengine_supported(int n) { return fengine_t2(n) > 0; }
 
 corr_status launch_fengine_range(const Handle &h, const void *volt, const float *scale, void *out, int i0, int n_run,
@@ -80,7 +79,7 @@ corr_status launch_fengine_range(const Handle &h, const void *volt, const float 
     f.i0 = i0;
     f.n_run = n_run;
     if (n_run == 0) return CORR_OK;
-    if (pfb_fused(h)) {
+    if (h.pfb_win && pfb_fused(h, h.pfb_taps)) {
         StageScope sc(h, CORR_STAGE_FENGINE, st);
         auto run = h.pfb_taps <= 4 ? fengine_run_pfb4 : fengine_run_pfb8;
         return run((h.flags & CORR_FLAG_PLANAR) != 0, f, h.pfb_win, h.pfb_taps, volt, scale, out, st);

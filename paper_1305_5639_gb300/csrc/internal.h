@@ -189,6 +189,8 @@ corr_status selftest_bounded_wait(uint64_t limit_ns);
 // Polyphase filter bank: FIR pass of inputs [i0, i0 + n_run) into h.pfb_y (pfb.cu).
 corr_status launch_pfb_fir(const Handle &h, const void *volt, int i0, int n_run, cudaStream_t st);
 bool fengine_supported(int n_chan);
+// Whether a window of `taps` taps is applied inside the F-engine (else by a FIR pass).
+bool pfb_fused(const Handle &h, int taps);
 // tensor-core F-engine (fengine_tc.cu): N = 1024, INT8, no delays or filter bank
 bool fengine_tc_applies(const Handle &h);
 corr_status fengine_tc_init(Handle &h);

@@ -41,3 +41,27 @@ def test_fused_filter_bank_equals_two_pass(cuda_ok, N, K, P, delays, planar):
     assert np.array_equal(codes.astype(np.float64), np.clip(np.rint(S), -127, 127) + 0.0)
     a.close()
     b.close()
+
+
+def test_power_pass_makes_its_frames_during_a_capture(cuda_ok):
+    """The fused filter bank needs no frame buffer; the power pass makes it when first
+    called, in a stream capture too, and its replays give the powers of the eager call."""
+    N, K, n_in = 256, 24, 4
+    v = torch.from_numpy(synth.volt_int8(n_in, 1, N, K, seed=8)).to(DEV)
+    h = np.random.default_rng(2).standard_normal((4, N)).astype(np.float32)
+    c = api.Correlator(n_in, 1, N, K, precision="int8")
+    c.set_pfb(h)
+    out = torch.zeros(N, device=DEV)
+    s = torch.cuda.Stream()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(s), torch.cuda.graph(g, stream=s):
+        c.fengine_power(v, out=out)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    d = api.Correlator(n_in, 1, N, K, precision="int8")
+    d.set_pfb(h)
+    want = d.fengine_power(v)
+    assert torch.allclose(out, want, rtol=1e-5) and bool((out > 0).all())
+    c.close()
+    d.close()
