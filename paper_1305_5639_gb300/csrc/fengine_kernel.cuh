@@ -295,9 +295,31 @@ __device__ __forceinline__ void dft_shared(const float2 (&lo)[L / 4], const floa
     fft_dif<L / 2, L / 2, 1, PACK>(v);
 }
 
+// CTAs per SM the register allocation aims at. The shorter transforms hold 8 or 16 values per
+// thread and wait on loads and barriers, so more warps in flight pay for as long as nothing
+// spills; the delay form, which converts its samples with synchronous loads, gains most.
+// 128 inputs, int8 layout, us (3 CTAs, or 2 at N = 512, before): delays N = 512 x 8192 spectra
+// 1252 -> 1101 with 4, N = 256 x 16384 1079 -> 1002 with 4, 951 with 5 and 1096 with 6, N =
+// 128 x 16384 661 -> 566 with 5, 547 with 6, N = 64 x 32768 597 -> 554 with 5, 537 with 6;
+// no delays N = 256 848 -> 842 with 4 (planar 952 -> 923), 849 with 5, N = 128 528 -> 503
+// with 5 and 504 with 6, N = 64 476 -> 453 with 6. FP32 voltages gain from 6 up to N = 128
+// (334 -> 313 for 8192 spectra) and nothing above. The filter bank keeps its FIR quads in
+// registers: more CTAs help at N = 64 only (4 taps 729 -> 669 with 6; 8 taps 935 -> 823 with
+// 4, 983 with 5).
+template <int N, bool I8, int MODE, int FEAT, int P>
+constexpr int fengine_ctas() {
+    if (N >= 2048) return FCfg<N, I8, MODE, FEAT>::NT == 512 ? 1 : 2;
+    if (MODE == kPower) return N >= 1024 ? 1 : N >= 512 ? 2 : 3;
+    if (N >= 1024) return 2;
+    if (FEAT == kPfb) return N >= 512 ? 2 : N != 64 ? 3 : P <= 4 ? 6 : 4;
+    if (N == 512) return I8 && FEAT == kDelay ? 4 : 2;
+    if (N == 256) return !I8 ? 3 : FEAT == kDelay ? 5 : 4;
+    if (N == 128) return I8 && FEAT == kPlain ? 5 : 6;
+    return N == 64 ? 6 : 3;
+}
+
 template <int N, bool I8, int MODE, int FEAT, int P = 0>
-__global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, N >= 2048 ? (FCfg<N, I8, MODE, FEAT>::NT == 512 ? 1 : 2)
-                                                               : (MODE == kPower && N >= 1024) ? 1 : (N >= 512 ? 2 : 3)) k_fengine(const void *__restrict__ volt,
+__global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I8, MODE, FEAT, P>()) k_fengine(const void *__restrict__ volt,
                                                       const float *__restrict__ scale,
                                                       void *__restrict__ out,
                                                       double *__restrict__ power, int n_in, int K,
