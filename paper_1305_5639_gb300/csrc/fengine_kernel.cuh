@@ -72,7 +72,9 @@ struct FCfg {
     // long re-packed transforms read the twiddles through L1 instead of a shared-memory copy,
     // so that two CTAs fit on an SM at N = 2048 (one's copy-out beside the other's FFTs: 370
     // -> 324 us below) and twice the staging rows at N = 4096
-    static constexpr bool TWG = N >= 2048 && RQ && FEAT != kPfb;
+    // (so does the power pass at N = 4096 without delays: 1344 -> 1263 us for 128 inputs x 1024
+    // spectra; 1560 -> 1803 with delays, whose phases then multiply every factor again)
+    static constexpr bool TWG = (N >= 2048 && RQ && FEAT != kPfb) || (N == 4096 && MODE == kPower && FEAT == kPlain);
     // threads per CTA: 256, or 512 where the shared memory leaves room for one CTA only
     static constexpr int NT = (N >= 2048 && RQ && !TWG) || (N == 4096 && RQ) ? 512 : 256;
     static constexpr int G = NT / TG;         // FFTs in flight per CTA
@@ -100,6 +102,11 @@ struct FCfg {
     // The long transforms may take fewer spectra per CTA than SB (see launch_one_); for the
     // others the variable loop bound cost more (1 to 4 %) than a fuller chip gains.
     static constexpr bool VARSB = RQ && N >= 2048;
+    // The power pass runs over many blocks of SB spectra per CTA (see launch_one_): its
+    // channel sums stay in shared memory as FP64, and a thread adds PQ of its spectra in
+    // FP32 before they join (no more roundings than the FP32 sum over a block of SB had).
+    static constexpr bool POW = MODE == kPower;
+    static constexpr int PQ = N == 2048 ? 5 : N == 512 || N == 1024 ? 6 : 8;
     // staging row stride in 32-bit words. The re-packing modes stage one 16-bit code
     // pair per (channel k, spectrum s): a row of SB / 2 words whose word index is
     // XOR-swizzled with (k >> SW) & (ROWW - 1), SW = log2(32 / ROWW), so that the
@@ -110,7 +117,7 @@ struct FCfg {
     static constexpr int SW = RQ ? ilog2(32 / ROWW) : 0;
     static_assert(!RQ || (ROWW >= 4 && ROWW <= 16), "swizzle assumes 4..16-word rows");
     static constexpr size_t ex_bytes = sizeof(float) * (size_t)G * GS;
-    static constexpr size_t pw_bytes = MODE == kPower ? sizeof(float) * N : 0;
+    static constexpr size_t pw_bytes = POW ? sizeof(double) * N : 0;  // FP64 channel sums
     static constexpr size_t tw_bytes = TWG ? 0 : sizeof(float2) * (size_t)N;  // twiddle table copy
     static constexpr size_t dl_bytes = sizeof(float2) * 64;         // delay phases d[k2] (T2 <= 64)
     static constexpr size_t st_bytes = sizeof(uint32_t) * (size_t)N * ROWW;
@@ -305,11 +312,11 @@ __device__ __forceinline__ void dft_shared(const float2 (&lo)[L / 4], const floa
 // with 5 and 504 with 6, N = 64 476 -> 453 with 6. FP32 voltages gain from 6 up to N = 128
 // (334 -> 313 for 8192 spectra) and nothing above. The filter bank keeps its FIR quads in
 // registers: more CTAs help at N = 64 only (4 taps 729 -> 669 with 6; 8 taps 935 -> 823 with
-// 4, 983 with 5).
+// 4, 983 with 5). The power pass has no staging rows: N = 1024 with delays 1604 -> 1104 with 2.
 template <int N, bool I8, int MODE, int FEAT, int P>
 constexpr int fengine_ctas() {
     if (N >= 2048) return FCfg<N, I8, MODE, FEAT>::NT == 512 ? 1 : 2;
-    if (MODE == kPower) return N >= 1024 ? 1 : N >= 512 ? 2 : 3;
+    if (MODE == kPower) return N == 1024 ? 2 : N >= 512 ? 3 : N == 256 ? 4 : 5;
     if (N >= 1024) return 2;
     if (FEAT == kPfb) return N >= 512 ? 2 : N != 64 ? 3 : P <= 4 ? 6 : 4;
     if (N == 512) return I8 && FEAT == kDelay ? 4 : 2;
@@ -348,7 +355,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
     const bool has_shift = DLY && dint != nullptr, has_dly = DLY && dph != nullptr;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *ex = reinterpret_cast<float *>(smem_raw);                                 // [G][T1][EXS]
-    float *scs = reinterpret_cast<float *>(smem_raw + C::ex_bytes);                  // [N] (power)
+    double *psum = reinterpret_cast<double *>(smem_raw + C::ex_bytes);               // [N] (power)
     float2 *tws = reinterpret_cast<float2 *>(smem_raw + C::ex_bytes + C::pw_bytes);  // [k1][t] twiddles
     float2 *dsm = reinterpret_cast<float2 *>(smem_raw + C::ex_bytes + C::pw_bytes + C::tw_bytes);  // [k2] phases
     uint32_t *stg = reinterpret_cast<uint32_t *>(smem_raw + C::ex_bytes + C::pw_bytes + C::tw_bytes +
@@ -364,7 +371,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
     };
 
     const int i = i0 + blockIdx.y;
-    const int sb = C::VARSB ? sb_run : SB;  // spectra per CTA
+    const int sb = C::VARSB || C::POW ? sb_run : SB;  // spectra per CTA
     const int a0 = blockIdx.x * sb;
     // Raw int8 frames without delays are copied asynchronously into the FFT's exchange
     // buffer (free between exchanges): the copy for the next frame is issued after the
@@ -391,19 +398,20 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
     // (it is common to thread k1's pass-2 DFT), d applied to the outputs.
     const long long n_rec = (long long)K * N;  // samples per input
     const int D = has_shift ? __ldg(dint + i) : 0;
-    {
-        // Warm L2 with this CTA's raw block (SB consecutive spectra of input i, one
-        // contiguous range): the loads of the later spectra then hit L2 instead of HBM.
+    // Warm L2 with the raw block of spectra [a_lo, a_hi) of input i (one contiguous range):
+    // the loads of the later spectra then hit L2 instead of HBM.
+    auto warm = [&](long long a_lo, long long a_hi) {
         constexpr int BPS = I8 ? 2 : 8;  // bytes per complex sample
-        const long long lo = max(0LL, (long long)a0 * N + D);
-        const long long hi = min(n_rec, (long long)min(K, a0 + sb) * N + D);
+        const long long lo = max(0LL, a_lo * N + D);
+        const long long hi = min(n_rec, min((long long)K, a_hi) * N + D);
         if (hi > lo) {
             const char *blk = reinterpret_cast<const char *>(volt) + ((size_t)i * n_rec + lo) * BPS;
             const int lines = (int)(((hi - lo) * BPS + 127) / 128);
             for (int l = threadIdx.x; l < lines; l += NT)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(blk + (size_t)l * 128));
         }
-    }
+    };
+    warm(a0, (long long)a0 + min(SB, sb));
     // per-CTA copy of the twiddle table (shared-memory loads in the FFT loop; measured
     // faster than L1 lookups, while the channel scales are faster from L1)
     const bool tw_async = PFB && !has_dly;  // as it stands: in flight while the first frames form
@@ -412,6 +420,9 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
         cp_async_commit();
     }
     if (C::TWG && has_dly && threadIdx.x < T2) dsm[threadIdx.x] = __ldg(dph + (size_t)i * (T1 + T2) + T1 + threadIdx.x);
+    if constexpr (C::POW) {
+        for (int m = threadIdx.x; m < N; m += NT) psum[m] = 0.0;
+    }
     for (int m = threadIdx.x; m < N && !tw_async && !C::TWG; m += NT) {
         float2 w = __ldg(tw_glob + m);
         if (DLY && has_dly) {
@@ -420,7 +431,6 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
         }
         if constexpr (SCALED) w = make_float2(w.x * (1.0f / kI8Scale), w.y * (1.0f / kI8Scale));
         tws[m] = w;
-        if constexpr (MODE == kPower) scs[m] = 0.0f;
     }
     if constexpr (!PFB) __syncthreads();
 
@@ -439,11 +449,13 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
         for (int q = 0; q < R2; ++q) pw[q] = 0.0f;
     }
 
-    for (int s0 = 0; s0 < SB; s0 += G) {
+    for (int s0 = 0; s0 < (C::POW ? sb : SB); s0 += G) {
         if (C::VARSB && s0 >= sb) break;  // (sb is a multiple of G)
+        if (C::POW && s0 % SB == 0) warm((long long)a0 + s0 + SB, a0 + min(s0 + 2LL * SB, (long long)sb));
+        const bool join = C::POW && ((s0 / G) % C::PQ == C::PQ - 1 || s0 + G >= sb);  // partial sums meet below
         const int s = s0 + g;
         const int a = a0 + s;
-        const bool valid = (s < SB) && (a < K);
+        const bool valid = (s < (C::POW ? sb : SB)) && (a < K);
         float2 v[TV];
         // ---- pass 1: column col takes x[col + T2 m]: value m of the R1 this thread holds is
         // sample mm(m) of the column
@@ -558,7 +570,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
                 hi[4 * j].y = b.x, hi[4 * j + 1].y = b.y, hi[4 * j + 2].y = b.z, hi[4 * j + 3].y = b.w;
             }
             group_sync();
-            if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
+            if (use_async && s0 + G < sb && !join) issue_raw(s0 + G + g);  // next frame into the free buffer
             dft_shared<T2, HB, PACK>(lo, hi, h2, v);  // v[bitrev(k')] = X[row + T1 k2], k2 = 2 k' + h2
         } else if constexpr (kScalarStage) {
             // the rows are read into plain float arrays (a 16-byte load fills four
@@ -585,7 +597,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
                 }
             }
             group_sync();
-            if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
+            if (use_async && s0 + G < sb && !join) issue_raw(s0 + G + g);  // next frame into the free buffer
             // pass 2: its first radix-2 stage in scalar arithmetic, from the float arrays
             // into the (re, im) pairs, then the remaining stages on the pairs
             sfor<0, T2 / 2>([&](auto J) {
@@ -620,7 +632,7 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
                 }
             }
             group_sync();
-            if (use_async && s0 + G < sb) issue_raw(s0 + G + g);  // next frame into the free buffer
+            if (use_async && s0 + G < sb && !join) issue_raw(s0 + G + g);  // next frame into the free buffer
             fft_dif<T2, TV, 0, PACK>(v);  // v[bitrev(k2)] = X[t + T1 k2]
         }
         if (PFB && has_dly) {
@@ -651,6 +663,38 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
                     pw[k2] += x.x * x.x + x.y * x.y;
                 }
             });
+        }
+        if (C::POW && join) {
+            // The FP32 sums of the FFTs that share a warp are added (shuffles), each FFT's
+            // lanes writing their share of the channels to the warp's part of the exchange
+            // buffer; then a thread per channel adds the warps' sums, and the result to the FP64
+            // sum (each warp's sum added in FP64: N = 1024, 16 inputs x 256 spectra 28.9 us
+            // against 22.5).
+            constexpr int FW = TG < 32 ? 32 / TG : 1, PARTS = G / FW;  // FFTs per warp; partial sums
+            const int fft = (threadIdx.x % 32) / TG;
+            float *part = ex + (size_t)(g / FW * FW) * C::GS;
+            sfor<0, R2>([&](auto K2) {
+                constexpr int k2 = decltype(K2)::value;
+                float p = pw[k2];
+#pragma unroll
+                for (int x = 1; x < FW; x *= 2) p += __shfl_xor_sync(0xffffffffu, p, x * TG);
+                if (FW == 1 || fft == k2 % FW) part[row + T1 * (H2 * k2 + h2)] = p;
+                pw[k2] = 0.0f;
+            });
+            __syncthreads();
+            for (int m = threadIdx.x; m < N; m += NT) {
+                float d[PARTS];
+#pragma unroll
+                for (int x = 0; x < PARTS; ++x) d[x] = ex[(size_t)(x * FW) * C::GS + m];
+#pragma unroll
+                for (int h = PARTS / 2; h > 0; h /= 2)
+#pragma unroll
+                    for (int x = 0; x < h; ++x) d[x] += d[x + h];
+                if (s0 + G < sb) psum[m] += (double)d[0];
+                else atomicAdd(&power[m], psum[m] + (double)d[0]);
+            }
+            __syncthreads();
+            if (use_async && s0 + G < sb) issue_raw(s0 + G + g);
         }
     }
 
@@ -727,15 +771,6 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
             }
         }
     }
-
-    if constexpr (MODE == kPower) {
-        sfor<0, R2>([&](auto K2) {
-            constexpr int k2 = decltype(K2)::value;
-            atomicAdd(&scs[row + T1 * (H2 * k2 + h2)], pw[k2]);
-        });
-        __syncthreads();
-        for (int m = threadIdx.x; m < N; m += NT) atomicAdd(&power[m], (double)scs[m]);
-    }
 }
 
 template <int N, bool I8, int MODE, int FEAT, int P = 0>
@@ -756,6 +791,20 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     const int n_rows = f.n_run < 0 ? f.n_in : f.n_run;
     int sb = C::SB;
     while (C::VARSB && sb / 2 >= C::G && sb / 2 >= 8 && (long long)((f.n_spectra + sb - 1) / sb) * n_rows < f.n_sm) sb /= 2;
+    // The power pass: blocks of SB spectra per CTA up to 2^16 samples, while 16 CTAs are left
+    // for each SM (a CTA ends with one FP64 atomic per channel, and atomics to one address take
+    // 16 ns each: with one CTA per block they were all the time of short transforms); parts
+    // of a block, whole rounds of the G FFTs in flight, while there are not two CTAs per SM
+    // (one at N = 4096, whose atomics weigh more: 16 inputs x 60 spectra 31.8 -> 27.8 us, but
+    // 36.3 with one CTA per block).
+    // 128 inputs, int8, us: N = 16 x 32768 spectra 1210 -> 103, N = 64 x 32768 2095 -> 338, N =
+    // 256 x 16384 2095 -> 662, N = 512 x 8192 2013 -> 815, N = 1024 x 4096 1318 -> 803, N =
+    // 2048 x 2048 1890 -> 1015, N = 4096 x 1024 1318 -> 1263.
+    if (C::POW) {
+        const long long blocks = (f.n_spectra + C::SB - 1) / C::SB, want = 16LL * f.n_sm;
+        sb *= (int)std::min(std::min(blocks, std::max(1LL, (1LL << 16) / (C::SB * N))), std::max(1LL, blocks * n_rows / want));
+        while (sb <= C::SB && sb / 2 >= C::G && (long long)((f.n_spectra + sb - 1) / sb) * n_rows < (N >= 4096 ? 1LL : 2LL) * f.n_sm) sb /= 2;
+    }
     dim3 grid((f.n_spectra + sb - 1) / sb, n_rows);
     // asynchronous raw copies need 16-byte aligned frames (2 N bytes each, N >= 64); the
     // public entry points only accept 16-byte aligned voltages, so this is a safeguard
