@@ -262,7 +262,9 @@ CORR_API corr_status corr_get_accum(corr_t *h, void *out, void *stream);
  * corr_xengine launch adds it to the FP64 buffer from warps that would otherwise
  * idle, overlapping the X-engine. corr_flush, corr_dump with vis_out and
  * corr_fx_host complete a deferred dump first, so every reader of the FP64
- * buffer sees the same sums as with an immediate dump (bit for bit). */
+ * buffer sees the same sums as with an immediate dump (bit for bit). One that waits
+ * when a call on the handle is recorded into a CUDA graph is completed, and waited
+ * for, before the recording, so that replays do not add it again. */
 CORR_API corr_status corr_dump(corr_t *h, double *vis_out, void *stream);
 
 /* Complete any deferred dump (see corr_dump) on `stream` now: afterwards the FP64

@@ -146,7 +146,9 @@ void free_buffers(Handle &h) {
     }
     cudaFree(h.acc_alt);
     h.acc_alt = nullptr;
-    h.dump_pending = false;
+    if (h.settled_ev) cudaEventDestroy(h.settled_ev);
+    h.settled_ev = nullptr;
+    h.dump_pending = h.pending_eager = false;
     h.pending_src = nullptr;
     h.acc = nullptr;
     h.vis64 = nullptr;
@@ -162,16 +164,26 @@ bool use_tc(const Handle &h) {
     return h.precision != CORR_PREC_FP32;  // FP32 has no tensor-core X-engine
 }
 
+// Lets this thread make calls that a stream capture elsewhere would refuse (allocations,
+// waits) for as long as it lives; they are not recorded.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    bool ok;
+    RelaxedCapture() { ok = cudaThreadExchangeStreamCaptureMode(&mode) == cudaSuccess; }
+    ~RelaxedCapture() {
+        if (ok) cudaThreadExchangeStreamCaptureMode(&mode);
+    }
+    RelaxedCapture(const RelaxedCapture &) = delete;
+    RelaxedCapture &operator=(const RelaxedCapture &) = delete;
+};
+
 // The FIR output buffer of the two-pass filter bank: one complex FP32 frame per (input,
 // spectrum). Made with the window where the F-engine takes two passes, else by the first
 // power pass (also during a stream capture, which a relaxed capture mode allows).
 corr_status pfb_frames_buffer(Handle &h) {
     if (h.pfb_y) return CORR_OK;
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    CORR_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
-    const cudaError_t e = cudaMalloc(&h.pfb_y, sizeof(float2) * (size_t)h.n_in * h.n_spectra * h.n_chan);
-    cudaThreadExchangeStreamCaptureMode(&mode);
-    if (e != cudaSuccess) {
+    const RelaxedCapture relaxed;
+    if (cudaMalloc(&h.pfb_y, sizeof(float2) * (size_t)h.n_in * h.n_spectra * h.n_chan) != cudaSuccess) {
         cudaGetLastError();
         h.pfb_y = nullptr;
         set_error_text("allocating the filter bank's frame buffer failed");
@@ -189,26 +201,66 @@ bool defer_ok(const Handle &h) {
            !(h.flags & CORR_FLAG_FUSED_DUMP) && tma_available() && !xengine_i8_small(h);
 }
 
-// Remembers whether any call was recorded into a graph.
-void note_capture(Handle &h, cudaStream_t st) {
-    if (h.captured) return;
-    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
-        cudaGetLastError();
-        h.captured = true;
-    } else if (c != cudaStreamCaptureStatusNone) {
-        h.captured = true;
-    }
-}
-
 // Complete a deferred dump now (the dump kernel on the pending accumulator).
 // out, if not null, also receives the long integration.
 corr_status flush_dump(Handle &h, cudaStream_t st, double2 *out = nullptr) {
     if (!h.dump_pending) return CORR_OK;
     h.vis_zero = false;
     const corr_status s = launch_dump_src(h, h.pending_src, out, st);
-    if (s == CORR_OK) h.dump_pending = false;
+    if (s == CORR_OK) h.dump_pending = h.pending_eager = false;
     return s;
+}
+
+// Eager calls leave two things to the X-engine launch that follows: clearing the
+// accumulator (it stores) and a deferred dump (it carries it). A captured launch runs
+// later or never, and each time it is replayed; so both are done here, before the first
+// call is recorded, on a stream of their own after the eager work on the buffers, and
+// waited for. Without it an eager X-engine call before the first replay added to sums that
+// a reset had dropped, and every replay added the deferred integration again.
+corr_status settle(Handle &h) {
+    if (!h.acc_stale && !h.pending_eager) return CORR_OK;
+    const RelaxedCapture relaxed;
+    cudaStream_t st = nullptr;
+    CORR_CUDA_TRY(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+    auto run = [&]() -> corr_status {
+        CORR_CUDA_TRY(cudaStreamWaitEvent(st, h.settled_ev, 0));
+        if (h.pending_eager) {
+            const corr_status s = flush_dump(h, st);
+            if (s != CORR_OK) return s;
+        }
+        if (h.acc_stale) CORR_CUDA_TRY(cudaMemsetAsync(h.acc, 0, (size_t)h.n_chan * h.n_base * 8, st));
+        CORR_CUDA_TRY(cudaStreamSynchronize(st));
+        h.acc_stale = false;
+        return CORR_OK;
+    };
+    const corr_status s = run();
+    cudaStreamDestroy(st);
+    return s;
+}
+
+// To be called before a call touches the accumulator or the long integration: notes
+// whether it is being recorded into a graph, and settles the handle if so.
+corr_status note_capture(Handle &h, cudaStream_t st) {
+    cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &c) != cudaSuccess) {
+        cudaGetLastError();
+        h.captured = h.capturing = true;  // (the legacy stream beside a capture: what follows reports it)
+        return CORR_OK;
+    }
+    h.capturing = c != cudaStreamCaptureStatusNone;
+    if (!h.capturing) return CORR_OK;
+    h.captured = true;
+    return settle(h);
+}
+
+// The accumulator counts as zero from here on: the next X-engine call stores. cleared: its
+// memory is zero as well.
+corr_status accum_is_zero(Handle &h, cudaStream_t st, bool cleared = false) {
+    h.acc_zero = true;
+    h.acc_spectra = 0;
+    h.acc_stale = !cleared && !h.capturing;
+    if (h.acc_stale || h.pending_eager) CORR_CUDA_TRY(cudaEventRecord(h.settled_ev, st));
+    return CORR_OK;
 }
 
 // Planar FP16 operands of the tensor-core X-engine: the caller's buffer itself
@@ -275,7 +327,10 @@ static corr_status fx_host_run(corr_t *c, const void *volt_host, const float *ch
     if (accum_out && (h.flags & CORR_FLAG_FUSED_DUMP)) return CORR_EUNSUPPORTED;  // no INT32 accumulator then
     corr::DeviceGuard dg(h.device);
     cudaStream_t st = corr::as_stream(stream);
-    corr::note_capture(h, st);
+    {
+        const corr_status s = corr::note_capture(h, st);
+        if (s != CORR_OK) return s;
+    }
     h.vis_zero = false;
     {
         const corr_status s = corr::flush_dump(h, st);  // this pipeline dumps per channel block itself
@@ -364,10 +419,8 @@ static corr_status fx_host_run(corr_t *c, const void *volt_host, const float *ch
     }
     CORR_CUDA_TRY(cudaEventRecord(ev[1 + NB + NC], h.fx_out));
     CORR_CUDA_TRY(cudaStreamWaitEvent(st, ev[1 + NB + NC], 0));
-    h.acc_zero = true;
-    h.acc_spectra = 0;
     h.fx_par = par ^ 1;
-    return CORR_OK;
+    return corr::accum_is_zero(h, st);
 }
 
 }  // namespace corr
@@ -457,7 +510,8 @@ corr_status corr_create(int32_t n_ant, int32_t n_pol, int32_t n_chan, int32_t n_
     const size_t acc_bytes = nvis * 8;  // int2 or float2
     bool ok = cudaMalloc(&h.acc, acc_bytes) == cudaSuccess && cudaMalloc(&h.vis64, nvis * sizeof(double2)) == cudaSuccess &&
               cudaMalloc(&h.status, 3 * sizeof(int32_t)) == cudaSuccess &&
-              cudaMalloc(&h.power64, sizeof(double) * (size_t)n_chan) == cudaSuccess;
+              cudaMalloc(&h.power64, sizeof(double) * (size_t)n_chan) == cudaSuccess &&
+              cudaEventCreateWithFlags(&h.settled_ev, cudaEventDisableTiming) == cudaSuccess;
     if (ok && corr::fengine_supported(n_chan)) ok = cudaMalloc(&h.twiddle, sizeof(float2) * (size_t)n_chan) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -653,22 +707,22 @@ corr_status corr_xengine(corr_t *c, const void *chan_in, const float *gains, voi
     corr::DeviceGuard dg(h.device);
     const bool store = h.acc_zero;
     const float2 *g = reinterpret_cast<const float2 *>(gains);
-    corr_status s;
     cudaStream_t st = corr::as_stream(stream);
-    corr::note_capture(h, st);
+    corr_status s = corr::note_capture(h, st);
+    if (s != CORR_OK) return s;
     if (h.dump_pending || (h.flags & CORR_FLAG_FUSED_DUMP)) h.vis_zero = false;
     if (corr::use_tc(h) && !corr::xengine_i8_small(h)) {
         corr::TcOperands op;
         s = corr::tc_operands(h, chan_in, st, op);
         // a deferred dump of the previous integration rides along in this launch
         if (s == CORR_OK) s = corr::launch_xengine_tma(h, op.planes, op.npl, g, op.row_scale, op.kstride, store, st);
-        if (s == CORR_OK) h.dump_pending = false;
+        if (s == CORR_OK) h.dump_pending = h.pending_eager = false;
     } else {
         s = corr::flush_dump(h, st);
         if (s == CORR_OK) s = corr::launch_xengine_cudacore(h, chan_in, g, store, st);
     }
     if (s == CORR_OK) {
-        h.acc_zero = false;
+        h.acc_zero = h.acc_stale = false;
         h.acc_spectra += h.n_spectra;
     }
     return s;
@@ -699,6 +753,8 @@ corr_status corr_get_accum(corr_t *c, void *out, void *stream) {
     Handle &h = c->h;
     if (h.flags & CORR_FLAG_FUSED_DUMP) return CORR_ESTATE;
     corr::DeviceGuard dg(h.device);
+    // (a recorded copy reads the memory whenever it is replayed: resets then clear it)
+    if (const corr_status s = corr::note_capture(h, corr::as_stream(stream)); s != CORR_OK) return s;
     const size_t bytes = (size_t)h.n_chan * h.n_base * 8;
     // after a dump (or reset) the accumulator is logically zero; its memory is only
     // overwritten by the next X-engine launch
@@ -713,7 +769,7 @@ corr_status corr_dump(corr_t *c, double *vis_out, void *stream) {
     Handle &h = c->h;
     corr::DeviceGuard dg(h.device);
     cudaStream_t st = corr::as_stream(stream);
-    corr::note_capture(h, st);
+    if (const corr_status s = corr::note_capture(h, st); s != CORR_OK) return s;
     // the dump writes the copy along with the sums, where its 16-byte stores are aligned
     double2 *out = corr::aligned16(vis_out) ? reinterpret_cast<double2 *>(vis_out) : nullptr;
     bool copied = false;
@@ -731,6 +787,7 @@ corr_status corr_dump(corr_t *c, double *vis_out, void *stream) {
                 h.pending_src = h.acc;
                 std::swap(h.acc, h.acc_alt);
                 h.dump_pending = true;
+                h.pending_eager = !h.capturing;
                 deferred = true;
             }
         }
@@ -742,8 +799,7 @@ corr_status corr_dump(corr_t *c, double *vis_out, void *stream) {
         }
         if (s != CORR_OK) return s;
     }
-    h.acc_zero = true;
-    h.acc_spectra = 0;
+    if (const corr_status s = corr::accum_is_zero(h, st); s != CORR_OK) return s;
     if (vis_out && !copied) {
         copied = h.dump_pending && out;
         corr_status s = corr::flush_dump(h, st, out);
@@ -763,14 +819,12 @@ corr_status corr_restore_vis(corr_t *c, const double *vis_in, void *stream) {
     corr::DeviceGuard dg(h.device);
     cudaStream_t st = corr::as_stream(stream);
     const size_t bytes = (size_t)h.n_chan * h.n_base * sizeof(double2);
-    corr::note_capture(h, st);
+    if (const corr_status s = corr::note_capture(h, st); s != CORR_OK) return s;
     h.vis_zero = false;
     if (vis_in) CORR_CUDA_TRY(cudaMemcpyAsync(h.vis64, vis_in, bytes, cudaMemcpyDeviceToDevice, st));
     else CORR_CUDA_TRY(cudaMemsetAsync(h.vis64, 0, bytes, st));
-    h.dump_pending = false;  // the buffer it would have added to is replaced
-    h.acc_zero = true;
-    h.acc_spectra = 0;
-    return CORR_OK;
+    h.dump_pending = h.pending_eager = false;  // the buffer it would have added to is replaced
+    return corr::accum_is_zero(h, st);
 }
 
 corr_status corr_flush(corr_t *c, void *stream) {
@@ -778,7 +832,7 @@ corr_status corr_flush(corr_t *c, void *stream) {
     if (!c) return CORR_EINVAL;
     Handle &h = c->h;
     corr::DeviceGuard dg(h.device);
-    corr::note_capture(h, corr::as_stream(stream));
+    if (const corr_status s = corr::note_capture(h, corr::as_stream(stream)); s != CORR_OK) return s;
     return corr::flush_dump(h, corr::as_stream(stream));
 }
 
@@ -872,18 +926,17 @@ corr_status corr_reset(corr_t *c, void *stream) {
     cudaStream_t st = corr::as_stream(stream);
     const size_t nvis = (size_t)h.n_chan * h.n_base;
     // The accumulator's memory need not be cleared (acc_zero: the next X-engine call stores
-    // over it, and readers see zeros), nor a long integration that nothing was added to
-    // since the last reset; a gain-calibration step resets twice and dumps never (24 bytes
-    // per visibility each time: 242 of 3050 us for 512 inputs x 256 channels x 1024
-    // spectra). With captured calls about, whose replays bypass these flags, both are.
-    corr::note_capture(h, st);
+    // over it, readers see zeros, and settle() clears it before a call is captured), nor a
+    // long integration that nothing was added to since the last reset; a gain-calibration
+    // step resets twice and dumps never (24 bytes per visibility each time: 242 of 3050 us
+    // for 512 inputs x 256 channels x 1024 spectra). With captured calls about, whose
+    // replays bypass these flags, both are.
+    if (const corr_status s = corr::note_capture(h, st); s != CORR_OK) return s;
     if (h.captured) CORR_CUDA_TRY(cudaMemsetAsync(h.acc, 0, nvis * 8, st));
     if (h.captured || !h.vis_zero) CORR_CUDA_TRY(cudaMemsetAsync(h.vis64, 0, nvis * sizeof(double2), st));
     h.vis_zero = true;
-    h.dump_pending = false;
-    h.acc_zero = true;
-    h.acc_spectra = 0;
-    return CORR_OK;
+    h.dump_pending = h.pending_eager = false;
+    return corr::accum_is_zero(h, st, h.captured);
 }
 
 corr_status corr_backward(corr_t *c, const float *grad_vis, const void *chan_in, const float *gains, float *grad_chan,

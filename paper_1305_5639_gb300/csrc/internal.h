@@ -47,6 +47,12 @@ struct Handle {
     bool vis_zero = false;       // vis64 known to be all-zero (zeroed by a reset, nothing added since)
     bool captured = false;       // a call on this handle was stream-captured: its replays may change
                                  // the buffers without the flags above knowing
+    bool capturing = false;      // the present call is being captured
+    // What eager calls left to the next X-engine launch, and so has to be made good when
+    // that launch is captured (settle in corr_api.cu): acc_zero while acc holds old sums, and
+    // a deferred dump; settled_ev follows the last eager work on those buffers
+    bool acc_stale = false, pending_eager = false;
+    cudaEvent_t settled_ev = nullptr;
     float2 *twiddle = nullptr;   // F-engine twiddles W_N^(t k1), [k1][t], N = T1 x T2
     void *ftc_b = nullptr;       // tensor-core F-engine DFT matrices F_h, F_l (N = 1024, INT8)
     int32_t *dly_int = nullptr;  // delay compensation (null: off): integer advance per input
