@@ -103,10 +103,17 @@ struct FCfg {
     // others the variable loop bound cost more (1 to 4 %) than a fuller chip gains.
     static constexpr bool VARSB = RQ && N >= 2048;
     // The power pass runs over many blocks of SB spectra per CTA (see launch_one_): its
-    // channel sums stay in shared memory as FP64, and a thread adds PQ of its spectra in
-    // FP32 before they join (no more roundings than the FP32 sum over a block of SB had).
+    // channel sums stay in shared memory as FP64. A thread adds PQ of its spectra in FP32 and
+    // the FW FFTs of a warp join in FP32, 16 spectra at most and 8 in a row, what an FP32 sum
+    // in order over 16 spectra may lose; the warps' sums join without a rounding.
+    // (Modelled with exponentially distributed powers, rms error against that sum's: 0.66 at
+    // N = 16, 0.68 at 64, 0.75 up to 256, 0.73 up to 1024, 0.83 above.)
     static constexpr bool POW = MODE == kPower;
-    static constexpr int PQ = N == 2048 ? 5 : N == 512 || N == 1024 ? 6 : 8;
+    static constexpr int FW = TG < 32 ? 32 / TG : 1;  // FFTs per warp
+    static constexpr int PQ = FW > 2 ? 16 / FW : 8;
+    // blocks of SB spectra per CTA at most, and whether they join more than once
+    static constexpr int POWB = N * SB < 1 << 16 ? (1 << 16) / (N * SB) : 1;
+    static constexpr bool PSUM = POW && POWB * SB > PQ * G;
     // staging row stride in 32-bit words. The re-packing modes stage one 16-bit code
     // pair per (channel k, spectrum s): a row of SB / 2 words whose word index is
     // XOR-swizzled with (k >> SW) & (ROWW - 1), SW = log2(32 / ROWW), so that the
@@ -117,7 +124,7 @@ struct FCfg {
     static constexpr int SW = RQ ? ilog2(32 / ROWW) : 0;
     static_assert(!RQ || (ROWW >= 4 && ROWW <= 16), "swizzle assumes 4..16-word rows");
     static constexpr size_t ex_bytes = sizeof(float) * (size_t)G * GS;
-    static constexpr size_t pw_bytes = POW ? sizeof(double) * N : 0;  // FP64 channel sums
+    static constexpr size_t pw_bytes = PSUM ? sizeof(double) * N : 0;  // FP64 channel sums
     static constexpr size_t tw_bytes = TWG ? 0 : sizeof(float2) * (size_t)N;  // twiddle table copy
     static constexpr size_t dl_bytes = sizeof(float2) * 64;         // delay phases d[k2] (T2 <= 64)
     static constexpr size_t st_bytes = sizeof(uint32_t) * (size_t)N * ROWW;
@@ -166,6 +173,13 @@ __device__ __forceinline__ void cp_async16(void *sdst, const void *gsrc) {
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// a + b rounded; err gains what the rounding left out (Knuth's two-sum, exact)
+__device__ __forceinline__ float add_err(float a, float b, float &err) {
+    const float s = a + b, bb = s - a;
+    err += (a - (s - bb)) + (b - bb);
+    return s;
+}
 
 // Polyphase filter-bank parameters of one launch (see pfb_frames).
 struct PfbArgs {
@@ -420,9 +434,6 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
         cp_async_commit();
     }
     if (C::TWG && has_dly && threadIdx.x < T2) dsm[threadIdx.x] = __ldg(dph + (size_t)i * (T1 + T2) + T1 + threadIdx.x);
-    if constexpr (C::POW) {
-        for (int m = threadIdx.x; m < N; m += NT) psum[m] = 0.0;
-    }
     for (int m = threadIdx.x; m < N && !tw_async && !C::TWG; m += NT) {
         float2 w = __ldg(tw_glob + m);
         if (DLY && has_dly) {
@@ -667,10 +678,11 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
         if (C::POW && join) {
             // The FP32 sums of the FFTs that share a warp are added (shuffles), each FFT's
             // lanes writing their share of the channels to the warp's part of the exchange
-            // buffer; then a thread per channel adds the warps' sums, and the result to the FP64
-            // sum (each warp's sum added in FP64: N = 1024, 16 inputs x 256 spectra 28.9 us
-            // against 22.5).
-            constexpr int FW = TG < 32 ? 32 / TG : 1, PARTS = G / FW;  // FFTs per warp; partial sums
+            // buffer; then a thread per channel adds the warps' sums as FP32 pairs of sum and
+            // error, and the result to the FP64 sum (each warp's sum added in FP64: N = 1024, 16
+            // inputs x 256 spectra 28.9 us against 23.0; two of them are two conversions and one
+            // add either way).
+            constexpr int FW = C::FW, PARTS = G / FW;  // FFTs per warp; partial sums
             const int fft = (threadIdx.x % 32) / TG;
             float *part = ex + (size_t)(g / FW * FW) * C::GS;
             sfor<0, R2>([&](auto K2) {
@@ -686,12 +698,21 @@ __global__ void __launch_bounds__(FCfg<N, I8, MODE, FEAT>::NT, fengine_ctas<N, I
                 float d[PARTS];
 #pragma unroll
                 for (int x = 0; x < PARTS; ++x) d[x] = ex[(size_t)(x * FW) * C::GS + m];
+                double sum;
+                if constexpr (PARTS == 2) {
+                    sum = (double)d[0] + (double)d[1];
+                } else {
+                    float err = 0.0f;
 #pragma unroll
-                for (int h = PARTS / 2; h > 0; h /= 2)
+                    for (int h = PARTS / 2; h > 0; h /= 2)
 #pragma unroll
-                    for (int x = 0; x < h; ++x) d[x] += d[x + h];
-                if (s0 + G < sb) psum[m] += (double)d[0];
-                else atomicAdd(&power[m], psum[m] + (double)d[0]);
+                        for (int x = 0; x < h; ++x) d[x] = add_err(d[x], d[x + h], err);
+                    // (the error of an infinite sum is no number)
+                    sum = (double)d[0] + (err == err ? (double)err : 0.0);
+                }
+                if (C::PSUM && s0 / G >= C::PQ) sum += psum[m];  // not the first time
+                if (C::PSUM && s0 + G < sb) psum[m] = sum;
+                else atomicAdd(&power[m], sum);
             }
             __syncthreads();
             if (use_async && s0 + G < sb) issue_raw(s0 + G + g);
@@ -797,12 +818,12 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     // of a block, whole rounds of the G FFTs in flight, while there are not two CTAs per SM
     // (one at N = 4096, whose atomics weigh more: 16 inputs x 60 spectra 31.8 -> 27.8 us, but
     // 36.3 with one CTA per block).
-    // 128 inputs, int8, us: N = 16 x 32768 spectra 1210 -> 103, N = 64 x 32768 2095 -> 338, N =
-    // 256 x 16384 2095 -> 662, N = 512 x 8192 2013 -> 815, N = 1024 x 4096 1318 -> 803, N =
-    // 2048 x 2048 1890 -> 1015, N = 4096 x 1024 1318 -> 1263.
+    // 128 inputs, int8, us: N = 16 x 32768 spectra 1213 -> 118, N = 64 x 32768 2094 -> 354, N =
+    // 256 x 16384 2095 -> 668, N = 512 x 8192 2018 -> 818, N = 1024 x 4096 1332 -> 728, N =
+    // 2048 x 2048 1891 -> 996, N = 4096 x 1024 1319 -> 1268.
     if (C::POW) {
         const long long blocks = (f.n_spectra + C::SB - 1) / C::SB, want = 16LL * f.n_sm;
-        sb *= (int)std::min(std::min(blocks, std::max(1LL, (1LL << 16) / (C::SB * N))), std::max(1LL, blocks * n_rows / want));
+        sb *= (int)std::min(std::min(blocks, (long long)C::POWB), std::max(1LL, blocks * n_rows / want));
         while (sb <= C::SB && sb / 2 >= C::G && (long long)((f.n_spectra + sb - 1) / sb) * n_rows < (N >= 4096 ? 1LL : 2LL) * f.n_sm) sb /= 2;
     }
     dim3 grid((f.n_spectra + sb - 1) / sb, n_rows);
