@@ -13,7 +13,7 @@
 // Square lengths (16, 64, 256, 1024) take one thread per column and per row. For T2 = 2 T1
 // (128, 512, 2048) two threads share each row's T2-point DFT, and for 64 x 64 (4096) each
 // column's and each row's (dft_shared): every thread is busy in both passes and holds at
-// most 32 values, so that 16 warps fit on an SM.
+// most 32 values, so that 16 warps fit on an SM (but FCfg::ONE).
 // A CTA handles one input and SB consecutive spectra; the outputs are staged in
 // shared memory as [channel][spectrum] so that every (channel, input) row segment
 // of SB spectra is written to global memory contiguously (the corner turn). Raw
@@ -64,19 +64,23 @@ struct FCfg {
     static constexpr int T2 = fengine_t2(N);  // pass-1 threads = pass-2 DFT length
     static constexpr int T1 = N / T2;         // pass-1 DFT length = pass-2 threads
     static_assert(T2 > 0 && T1 * T2 == N && T1 <= T2 && T2 <= 64, "unsupported F-engine length");
-    static constexpr int H1 = T1 == 64 ? 2 : 1;             // threads per column in pass 1
-    static constexpr int H2 = T2 == 2 * T1 || T1 == 64 ? 2 : 1;  // threads per row in pass 2
+    // The power pass at N = 4096 without delays has no staging rows, and 64 values per thread
+    // fit its registers: one thread per DFT, in CTAs of two FFTs, two to an SM, beats shared
+    // DFTs in CTAs of 256 threads (int8, us: 128 inputs x 1024 spectra 1268 -> 1002, 16 x 256
+    // 65.7 -> 53.2, 16 x 128 41.1 -> 34.1; FP32 16 x 128 45.2 -> 36.0; with delays 1471 -> 1873:
+    // those share).
+    static constexpr bool ONE = N == 4096 && MODE == kPower && FEAT == kPlain;
+    static constexpr int H1 = T1 == 64 && !ONE ? 2 : 1;               // threads per column in pass 1
+    static constexpr int H2 = T2 == 2 * T1 || (T1 == 64 && !ONE) ? 2 : 1;  // threads per row in pass 2
     static constexpr int TG = T2 * H1;        // threads per FFT group
     static_assert(TG == T1 * H2, "every thread takes part in both passes");
     static constexpr bool RQ = MODE == kRequant || MODE == kRequantPlanar;
     // long re-packed transforms read the twiddles through L1 instead of a shared-memory copy,
     // so that two CTAs fit on an SM at N = 2048 (one's copy-out beside the other's FFTs: 370
     // -> 324 us below) and twice the staging rows at N = 4096
-    // (so does the power pass at N = 4096 without delays: 1344 -> 1263 us for 128 inputs x 1024
-    // spectra; 1560 -> 1803 with delays, whose phases then multiply every factor again)
-    static constexpr bool TWG = (N >= 2048 && RQ && FEAT != kPfb) || (N == 4096 && MODE == kPower && FEAT == kPlain);
+    static constexpr bool TWG = N >= 2048 && RQ && FEAT != kPfb;
     // threads per CTA: 256, or 512 where the shared memory leaves room for one CTA only
-    static constexpr int NT = (N >= 2048 && RQ && !TWG) || (N == 4096 && RQ) ? 512 : 256;
+    static constexpr int NT = (N >= 2048 && RQ && !TWG) || (N == 4096 && RQ) ? 512 : ONE ? 128 : 256;
     static constexpr int G = NT / TG;         // FFTs in flight per CTA
     // Exchange buffer of one FFT: T1 rows of EXS floats; row k1 receives Y[0..T2-1][k1]
     // (one column per writing thread) and is read back as float4. EXS and the per-FFT
@@ -816,11 +820,11 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     // for each SM (a CTA ends with one FP64 atomic per channel, and atomics to one address take
     // 16 ns each: with one CTA per block they were all the time of short transforms); parts
     // of a block, whole rounds of the G FFTs in flight, while there are not two CTAs per SM
-    // (one at N = 4096, whose atomics weigh more: 16 inputs x 60 spectra 31.8 -> 27.8 us, but
+    // (one at N = 4096, whose atomics weigh more: 16 inputs x 60 spectra, shared DFTs, 31.8 -> 27.8 us, but
     // 36.3 with one CTA per block).
     // 128 inputs, int8, us: N = 16 x 32768 spectra 1213 -> 118, N = 64 x 32768 2094 -> 354, N =
     // 256 x 16384 2095 -> 668, N = 512 x 8192 2018 -> 818, N = 1024 x 4096 1332 -> 728, N =
-    // 2048 x 2048 1891 -> 996, N = 4096 x 1024 1319 -> 1268.
+    // 2048 x 2048 1891 -> 996, N = 4096 x 1024 1319 -> 1002.
     if (C::POW) {
         const long long blocks = (f.n_spectra + C::SB - 1) / C::SB, want = 16LL * f.n_sm;
         sb *= (int)std::min(std::min(blocks, (long long)C::POWB), std::max(1LL, blocks * n_rows / want));
