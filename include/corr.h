@@ -172,7 +172,9 @@ CORR_API corr_status corr_set_delays(corr_t *h, const float *delays);
  * a of input i, the frame y[n] = sum_p h[p][n] s'_i[(a + p) n_chan + n] (s'_i the
  * stream after any delay compensation, zero past the record, so each input keeps
  * n_spectra spectra; with delays the per-channel phase follows the transform).
- * Synchronises the device. CORR_EUNSUPPORTED when n_chan has no F-engine,
+ * For float voltages, more than 8 taps or n_chan = 16 the frames take a buffer, 8 bytes
+ * per sample, that this call allocates (CORR_ENOMEM leaves the filter bank off); the
+ * other windows need none. Synchronises the device. CORR_EUNSUPPORTED when n_chan has no F-engine,
  * CORR_EINVAL for a bad tap count or a non-finite weight. */
 CORR_API corr_status corr_set_pfb(corr_t *h, int32_t n_taps, const float *window);
 

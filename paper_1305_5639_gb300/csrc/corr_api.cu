@@ -177,21 +177,6 @@ struct RelaxedCapture {
     RelaxedCapture &operator=(const RelaxedCapture &) = delete;
 };
 
-// The FIR output buffer of the two-pass filter bank: one complex FP32 frame per (input,
-// spectrum). Made with the window where the F-engine takes two passes, else by the first
-// power pass (also during a stream capture, which a relaxed capture mode allows).
-corr_status pfb_frames_buffer(Handle &h) {
-    if (h.pfb_y) return CORR_OK;
-    const RelaxedCapture relaxed;
-    if (cudaMalloc(&h.pfb_y, sizeof(float2) * (size_t)h.n_in * h.n_spectra * h.n_chan) != cudaSuccess) {
-        cudaGetLastError();
-        h.pfb_y = nullptr;
-        set_error_text("allocating the filter bank's frame buffer failed");
-        return CORR_ENOMEM;
-    }
-    return CORR_OK;
-}
-
 // Integration dumps are deferred into the next X-engine launch, whose warps run them
 // beside the MMAs (see corr_dump and SideDump in xengine_tma.cu): INT8 and FP16 hi/lo on
 // the tensor cores. Plain FP16 dumps at once, so that its calls can be captured and
@@ -626,9 +611,13 @@ corr_status corr_set_pfb(corr_t *c, int32_t n_taps, const float *window) {
     cudaFree(h.pfb_win);
     h.pfb_win = nullptr;
     h.pfb_taps = 0;
-    if (!corr::pfb_fused(h, n_taps)) {
-        const corr_status s = corr::pfb_frames_buffer(h);
-        if (s != CORR_OK) return s;
+    // the FIR output buffer of the two-pass filter bank: one complex FP32 frame per (input,
+    // spectrum); a fused one needs none
+    const size_t y_bytes = sizeof(float2) * (size_t)h.n_in * h.n_spectra * h.n_chan;
+    if (!corr::pfb_fused(h, n_taps) && !h.pfb_y && cudaMalloc(&h.pfb_y, y_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        h.pfb_y = nullptr;
+        return CORR_ENOMEM;
     }
     if (cudaMalloc(&h.pfb_win, sizeof(float) * n) != cudaSuccess) {
         cudaGetLastError();
@@ -687,10 +676,6 @@ corr_status corr_fengine_power(corr_t *c, const void *volt, float *power, void *
     if (!corr::fengine_supported(h.n_chan)) return CORR_EUNSUPPORTED;
     if (!corr::aligned16(volt)) return CORR_EINVAL;
     corr::DeviceGuard dg(h.device);
-    if (h.pfb_win) {
-        const corr_status s = corr::pfb_frames_buffer(h);
-        if (s != CORR_OK) return s;
-    }
     return corr::launch_fengine_power(h, volt, power, corr::as_stream(stream));
 }
 

@@ -46,10 +46,13 @@ __global__ void k_power_finalize(const double *__restrict__ p64, float *__restri
     if (k < n) out[k] = (float)(p64[k] * inv);
 }
 
-// Per-channel power: zero the FP64 accumulators, run the FFT pass, scale to a mean.
-corr_status power_pass(const FShape &f, const void *volt, double *acc64, float *power, cudaStream_t st) {
+// Per-channel power: zero the FP64 accumulators, run the FFT pass (with a window in pfb the
+// one that filters by itself), scale to a mean.
+corr_status power_pass(const FShape &f, const void *volt, double *acc64, float *power, cudaStream_t st,
+                       const PfbArgs &pfb = {}) {
     CORR_CUDA_TRY(cudaMemsetAsync(acc64, 0, sizeof(double) * f.n_chan, st));
-    corr_status s = dispatch<kPower>(f, volt, nullptr, nullptr, acc64, st);
+    const corr_status s = pfb.win ? fengine_run_pfb_power(f, pfb.win, pfb.taps, volt, acc64, st)
+                                  : dispatch<kPower>(f, volt, nullptr, nullptr, acc64, st);
     if (s != CORR_OK) return s;
     const double inv = 1.0 / (2.0 * (double)f.n_in * (double)f.n_spectra);
     k_power_finalize<<<(f.n_chan + 255) / 256, 256, 0, st>>>(acc64, power, f.n_chan, inv);
@@ -58,12 +61,13 @@ corr_status power_pass(const FShape &f, const void *volt, double *acc64, float *
 
 }  // namespace
 
-// Up to 8 taps on int8 voltages with re-packed output, the filter bank is fused into the
-// F-engine (pfb_frames): the FIR pass wrote 8 bytes per sample and the FFT read them back.
+// Up to 8 taps on int8 voltages the filter bank is fused into the F-engine (pfb_frames), its
+// power pass included: the FIR pass wrote 8 bytes per sample and the FFT read them back.
 // 128 inputs x 2 M samples, 4 taps: N = 1024 1361 -> 893 us, N = 256 1101 -> 648, N = 4096
-// 2107 -> 1597; 8 taps at N = 1024 1784 -> 1043. Longer windows (registers per thread), float
-// voltages and the power pass keep the two passes, as does N = 16 (fewer positions than
-// threads).
+// 2107 -> 1597; 8 taps at N = 1024 1784 -> 1043. The power pass, which then needs no buffer for
+// the frames (8 bytes per sample), 4 taps: N = 1024 1018 -> 679, N = 256 921 -> 498, N = 4096
+// 1426 -> 1036; 16 inputs x 256 spectra at N = 1024 45 -> 29. Longer windows (registers per
+// thread) and float voltages keep the two passes, as does N = 16 (fewer positions than threads).
 bool pfb_fused(const Handle &h, int taps) { return h.precision == CORR_PREC_INT8 && taps <= 8 && h.n_chan >= 64; }
 
 bool fengine_supported(int n) { return fengine_t2(n) > 0; }
@@ -101,6 +105,10 @@ corr_status launch_fengine(const Handle &h, const void *volt, const float *scale
 
 corr_status launch_fengine_power(const Handle &h, const void *volt, float *power, cudaStream_t st) {
     FShape f = shape_of(h);
+    if (h.pfb_win && pfb_fused(h, h.pfb_taps)) {
+        StageScope sc(h, CORR_STAGE_POWER, st, 2);
+        return power_pass(f, volt, h.power64, power, st, PfbArgs{h.pfb_win, h.pfb_taps});
+    }
     corr_status s = pfb_front(h, f, volt, st);
     if (s != CORR_OK) return s;
     StageScope sc(h, CORR_STAGE_POWER, st, 2);

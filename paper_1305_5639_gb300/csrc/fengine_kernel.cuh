@@ -22,8 +22,9 @@
 // 256 on an offset that the first butterflies cancel (i8_to_f2_scaled).
 //
 // This header holds the kernel template; the per-feature translation units
-// (fengine_plain.cu, fengine_delay.cu) instantiate it, so that the instantiations
-// compile in parallel, and fengine.cu holds the host entry points.
+// (fengine_plain.cu, fengine_delay.cu, fengine_pfb4.cu, fengine_pfb8.cu,
+// fengine_pfb_power.cu) instantiate it, so that the instantiations compile in
+// parallel, and fengine.cu holds the host entry points.
 #pragma once
 
 #include <algorithm>
@@ -334,7 +335,7 @@ __device__ __forceinline__ void dft_shared(const float2 (&lo)[L / 4], const floa
 template <int N, bool I8, int MODE, int FEAT, int P>
 constexpr int fengine_ctas() {
     if (N >= 2048) return FCfg<N, I8, MODE, FEAT>::NT == 512 ? 1 : 2;
-    if (MODE == kPower) return N == 1024 ? 2 : N >= 512 ? 3 : N == 256 ? 4 : 5;
+    if (MODE == kPower && FEAT != kPfb) return N == 1024 ? 2 : N >= 512 ? 3 : N == 256 ? 4 : 5;
     if (N >= 1024) return 2;
     if (FEAT == kPfb) return N >= 512 ? 2 : N != 64 ? 3 : P <= 4 ? 6 : 4;
     if (N == 512) return I8 && FEAT == kDelay ? 4 : 2;
@@ -881,6 +882,24 @@ corr_status launch_pfb(bool planar, const FShape &f, const PfbArgs &pfb, const v
 #undef CORR_F_CASE
 }
 
+// The power pass of the fused filter bank of up to P taps.
+template <int P>
+corr_status launch_pfb_power(const FShape &f, const PfbArgs &pfb, const void *volt, double *power, cudaStream_t st) {
+#define CORR_F_CASE(NN) \
+    case NN: return launch_one_<NN, true, kPower, kPfb, P>(f, volt, nullptr, nullptr, power, st, pfb);
+    switch (f.n_chan) {
+        CORR_F_CASE(64)
+        CORR_F_CASE(128)
+        CORR_F_CASE(256)
+        CORR_F_CASE(512)
+        CORR_F_CASE(1024)
+        CORR_F_CASE(2048)
+        CORR_F_CASE(4096)
+        default: return CORR_EUNSUPPORTED;
+    }
+#undef CORR_F_CASE
+}
+
 // Every (mode, n_chan, input type) of one front-end feature.
 template <int FEAT>
 corr_status launch_feature(int mode, const FShape &f, const void *volt, const float *scale, void *out,
@@ -906,5 +925,7 @@ corr_status fengine_run_pfb4(bool planar, const FShape &f, const float *win, int
                              const float *scale, void *out, cudaStream_t st);
 corr_status fengine_run_pfb8(bool planar, const FShape &f, const float *win, int taps, const void *volt,
                              const float *scale, void *out, cudaStream_t st);
+corr_status fengine_run_pfb_power(const FShape &f, const float *win, int taps, const void *volt, double *power,
+                                  cudaStream_t st);
 
 }  // namespace corr

@@ -59,7 +59,7 @@ struct Handle {
     float2 *dly_ph = nullptr;    //   and phase tables [n_in][T1 + T2]: exp(+j 2 pi k1 f / N), exp(+j 2 pi T1 k2 f / N)
     float *pfb_win = nullptr;    // polyphase filter-bank window [pfb_taps][n_chan] (null: off)
     int32_t pfb_taps = 0;
-    void *pfb_y = nullptr;       //   its FIR output, complex FP32 [n_in][n_spectra][n_chan]
+    void *pfb_y = nullptr;       //   FIR output of the two-pass form, complex FP32 [n_in][n_spectra][n_chan]
     int32_t *st_out = nullptr;   // short-time visibilities (caller's buffer; null: off)
     int32_t st_block = 0;        //   spectra per block
     int32_t *status = nullptr;   // device status word (0 ok, else CORR_* code set by a kernel), then the
@@ -195,7 +195,8 @@ corr_status selftest_bounded_wait(uint64_t limit_ns);
 // Polyphase filter bank: FIR pass of inputs [i0, i0 + n_run) into h.pfb_y (pfb.cu).
 corr_status launch_pfb_fir(const Handle &h, const void *volt, int i0, int n_run, cudaStream_t st);
 bool fengine_supported(int n_chan);
-// Whether a window of `taps` taps is applied inside the F-engine (else by a FIR pass).
+// Whether a window of `taps` taps is applied inside the F-engine and its power pass (else by
+// a FIR pass).
 bool pfb_fused(const Handle &h, int taps);
 // tensor-core F-engine (fengine_tc.cu): N = 1024, INT8, no delays or filter bank
 bool fengine_tc_applies(const Handle &h);
