@@ -255,7 +255,8 @@ CORR_API corr_status corr_get_accum(corr_t *h, void *out, void *stream);
 
 /* Integration dump: vis64 += accumulator (FP64), accumulator = 0. If vis_out is
  * not NULL, the FP64 long-integration buffer is copied to it
- * ([n_chan][B] complex double, device). Asynchronous. The paper writes each
+ * ([n_chan][B] complex double, device; the dump itself writes it where it lies in the
+ * handle's device's memory, 16-byte aligned, else a copy). Asynchronous. The paper writes each
  * accumulation's visibilities out (Section 5, Section 6.3); the FP64 long
  * integration is this library's own addition, with no passage behind it.
  * On the INT8 and FP16_HILO tensor-core X-engine (without CORR_FLAG_FUSED_DUMP) a

@@ -159,6 +159,17 @@ void free_buffers(Handle &h) {
     free_clock(h);
 }
 
+// Whether p lies in memory of this device itself. Kernels store to such memory only: another
+// device's may be out of their reach, where a copy still gets there.
+bool on_device(const void *p, int device) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == device;
+}
+
 bool use_tc(const Handle &h) {
     if (h.xengine == CORR_XENG_CUDACORE) return false;
     return h.precision != CORR_PREC_FP32;  // FP32 has no tensor-core X-engine
@@ -755,8 +766,10 @@ corr_status corr_dump(corr_t *c, double *vis_out, void *stream) {
     corr::DeviceGuard dg(h.device);
     cudaStream_t st = corr::as_stream(stream);
     if (const corr_status s = corr::note_capture(h, st); s != CORR_OK) return s;
-    // the dump writes the copy along with the sums, where its 16-byte stores are aligned
-    double2 *out = corr::aligned16(vis_out) ? reinterpret_cast<double2 *>(vis_out) : nullptr;
+    // the dump writes the copy along with the sums, where its 16-byte stores are aligned and
+    // within reach
+    double2 *out = vis_out && corr::aligned16(vis_out) && corr::on_device(vis_out, h.device)
+                       ? reinterpret_cast<double2 *>(vis_out) : nullptr;
     bool copied = false;
     if (!h.acc_zero && !(h.flags & CORR_FLAG_FUSED_DUMP)) {
         corr_status s = CORR_OK;
