@@ -71,8 +71,9 @@ enum {
  * X-engine reads planar FP16 operands by TMA: the caller's own (CORR_FLAG_PLANAR)
  * or ones the library converts the input into, in a workspace allocated on first
  * use (4 bytes per complex sample, 8 for FP16_HILO). CUDACORE with INT8 uses exact
- * dp4a integer arithmetic, and so does AUTO for complex int8 data of up to 32 inputs (24
- * with an odd number of spectra), where it is the faster one; the results are the same. */
+ * dp4a integer arithmetic, and so does AUTO for complex int8 data of few inputs, where it is
+ * the faster one: up to 32 if n_spectra is a multiple of 8, down to 16 for many spectra of
+ * an odd number; the results are the same. */
 enum { CORR_XENG_AUTO = 0, CORR_XENG_CUDACORE = 1, CORR_XENG_TCGEN05 = 2 };
 
 /* Layout flags (corr_opts.flags).

@@ -131,7 +131,8 @@ struct DeviceGuard {
 };
 
 // Raises the dynamic shared memory limit of kernel Kern on the current device to `bytes`,
-// once per device (the attribute stays; it was set before every launch, 0.5 us each).
+// once per device (the attribute stays, through cudaDeviceReset and for other contexts on the
+// device too, as tried; it was set before every launch, 0.5 us each).
 template <auto Kern>
 corr_status allow_smem(int bytes) {
     static std::atomic<unsigned long long> done{0};  // devices 0 .. 63

@@ -448,10 +448,20 @@ __global__ void __launch_bounds__(NTH) k_xeng_i8(const char2 *__restrict__ X, in
 }  // namespace
 
 bool xengine_i8_small(const Handle &h) {
-    // (an odd number of spectra leaves single-spectrum loads: 32 inputs, 1024 channels, 1001
-    // spectra take 193 us here, 135 on the tensor cores; the work falls with the pairs)
-    return h.precision == CORR_PREC_INT8 && h.xengine == CORR_XENG_AUTO &&
-           h.n_in <= (h.n_spectra % 2 == 0 ? kSmallIn : 24) && !(h.flags & (CORR_FLAG_PLANAR | CORR_FLAG_FUSED_DUMP));
+    if (h.precision != CORR_PREC_INT8 || h.xengine != CORR_XENG_AUTO ||
+        (h.flags & (CORR_FLAG_PLANAR | CORR_FLAG_FUSED_DUMP)))
+        return false;
+    // Where the two sides measure equal (X-engine with dump, us, here / tensor cores, 64 and
+    // 1024 channels): 16-byte loads win up to 32 inputs (32 x 4000 spectra 39 / 60 and 235 /
+    // 438). 4-byte loads win up to 28 inputs (28 x 4002: 57 / 60, 412 / 421), above that up to
+    // 1000 spectra (32 x 1002: 25 / 25, 117 / 122; 32 x 4002: 68 / 60, 524 / 438). Single
+    // spectra win up to 16 inputs (16 x 4001: 45 / 58, 319 / 379), up to 20 for 1500 spectra
+    // (20 x 1001: 24 / 24, 95 / 112; 20 x 4001: 65 / 60, 455 / 399), up to 24 for 500 (24 x 401:
+    // 17 / 19, 60 / 62; 24 x 1001: 28 / 25, 126 / 115; 24 x 4001: 81 / 60, 604 / 419).
+    const int n = h.n_in, K = h.n_spectra;
+    if (K % 8 == 0) return n <= kSmallIn;
+    if (K % 2 == 0) return n <= 28 || (n <= kSmallIn && K <= 1000);
+    return n <= 16 || (n <= 20 && K <= 1500) || (n <= 24 && K < 500);
 }
 
 corr_status launch_xengine_cudacore(const Handle &h, const void *chan_in, const float2 *gains, bool store,
