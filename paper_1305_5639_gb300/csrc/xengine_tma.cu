@@ -590,19 +590,32 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
             const int chan = itm.chan;
             const int I0 = itm.bi * TILE, J0 = itm.bj * TILE;
             const int i = I0 + wq * 32 + lane;  // this lane's row while staging
-            if (!tc::mbar_wait(accf_bar(0), af_phase, abort_flag, p.status)) break;
+            // triangle: rows i < n_in, columns j <= i of the packed accumulator (or the FP64
+            // buffer); rectangle: rows i < n_p of group P, columns j < n_q of group Q. The
+            // factors of this lane's row and of column `lane` of the warp's 32 are read while the
+            // MMAs run and pass between the lanes by shuffles; read per column in the drain, as
+            // before, each piece of it waited for them (with dump, 16 inputs x 256 channels x 33
+            // spectra 31.0 -> 30.3 us, 130 x 256 x 401 123 -> 119, 130 x 512 x 1001 hi/lo 506 -> 499)
+            const int gi0 = p.rect ? p.p0 : 0, gj0 = p.rect ? p.q0 : 0;
+            const bool row = i < (p.rect ? p.n_p : itm.n_in);
+            const int jl = min(J0 + 32 * qc + lane, (p.rect ? p.n_q : itm.n_in) - 1);  // clamped: unused past the end
+            float2 gi = make_float2(1.f, 0.f), gj = gi;
+            if (p.gains) {
+                if (row) gi = __ldg(p.gains + gi0 + i);
+                gj = __ldg(p.gains + gj0 + jl);
+            }
+            // the operands' range scaling: V_ij carries 2^e_i 2^e_j, undone here (exact)
+            const float *rs = p.rsc ? p.rsc + (long long)chan * p.n_in : nullptr;
+            float si = 1.f, sj = 1.f;
+            if (rs) {
+                if (row) si = __ldg(rs + gi0 + i);
+                sj = __ldg(rs + gj0 + jl);
+            }
+            // (all lanes go on, or none: the factors pass between them)
+            if (!__all_sync(0xffffffffu, tc::mbar_wait(accf_bar(0), af_phase, abort_flag, p.status))) break;
             af_phase ^= 1u;
             tc::tc_fence_after();
             const uint32_t d = tmem + lane_off + (uint32_t)(32 * qc);
-            // triangle: rows i < n_in, columns j <= i of the packed accumulator (or the FP64
-            // buffer); rectangle: rows i < n_p of group P, columns j < n_q of group Q
-            const int gi0 = p.rect ? p.p0 : 0, gj0 = p.rect ? p.q0 : 0;
-            float2 gi = make_float2(1.f, 0.f);
-            if (p.gains && i < (p.rect ? p.n_p : itm.n_in)) gi = __ldg(p.gains + gi0 + i);
-            // the operands' range scaling: V_ij carries 2^e_i 2^e_j, undone here (exact)
-            const float *rs = p.rsc ? p.rsc + (long long)chan * p.n_in : nullptr;
-            float si = 1.f;
-            if (rs && i < (p.rect ? p.n_p : itm.n_in)) si = __ldg(rs + gi0 + i);
             // the tile's sums into registers first, so that the MMAs of the next tile wait for
             // the reads only, not for the scaling and the writes below (plain FP16, 2048 inputs
             // x 16 channels x 2048 spectra: 403 -> 379 us; hi/lo, three times the MMAs per
@@ -630,14 +643,14 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
 #pragma unroll
                 for (int x = 0; x < 8; ++x) {
                     float2 v = make_float2(V[8 * cb + x], V[32 + 8 * cb + x]);
-                    const int jg = min(jb + x, (p.rect ? p.n_q : itm.n_in) - 1);  // clamped: unused past the end
                     if (rs) {
-                        const float sij = si * __ldg(rs + gj0 + jg);
+                        const float sij = si * __shfl_sync(0xffffffffu, sj, 8 * cb + x);
                         v = make_float2(v.x * sij, v.y * sij);
                     }
                     if (p.gains) {
-                        const float2 gj = __ldg(p.gains + gj0 + jg);
-                        const float2 w = make_float2(gi.x * gj.x + gi.y * gj.y, gi.y * gj.x - gi.x * gj.y);
+                        const float gx = __shfl_sync(0xffffffffu, gj.x, 8 * cb + x);
+                        const float gy = __shfl_sync(0xffffffffu, gj.y, 8 * cb + x);
+                        const float2 w = make_float2(gi.x * gx + gi.y * gy, gi.y * gx - gi.x * gy);
                         v = make_float2(v.x * w.x - v.y * w.y, v.x * w.y + v.y * w.x);
                     }
                     sl[lane * 8 + ((x + (lane >> 1)) & 7)] = v;
@@ -718,7 +731,7 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
                     tc::tmem_ld8(d + 8u * cb, u);         // ar br
                     tc::tmem_ld8(d + 384u + 8u * cb, w);  // ai bi
                     tc::tmem_wait_ld();
-add_sums<false>(R + 8 * cb, u, w);
+                    add_sums<false>(R + 8 * cb, u, w);
                     tc::tmem_ld8(d + 256u + 8u * cb, u);  // ai br
                     tc::tmem_ld8(d + 128u + 8u * cb, w);  // ar bi
                     tc::tmem_wait_ld();
