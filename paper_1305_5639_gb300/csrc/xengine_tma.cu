@@ -127,7 +127,7 @@ struct TParams {
     const void *side_src;
     double2 *side_dst;
     long long side_n;
-    unsigned *side_ctr;  // chunks claimed, CTAs finished (both zero between launches)
+    unsigned *side_ctr;  // chunks claimed, CTAs finished (both zero between launches); null: fixed shares
 };
 
 // Everything a role needs to know about one work item.
@@ -278,8 +278,9 @@ __device__ __forceinline__ void write_sums16(const int (&R)[64], const Item &itm
 // of few spectra (250 inputs, 128 channels, 1504 spectra: 118 us; 91 with all warps and a
 // fixed slice per CTA; 81 with the counter; 68 without a dump; 128 inputs, 512 channels, 256
 // spectra: 119, 64, 59 and 32). The last CTA to finish clears the counters for the next
-// launch. The sums are exact (integer values below 2^53 for INT8; the FP64 add of the FP32
-// sums for FP16), as the dump kernel's.
+// launch. A small dump goes to warps 2 and 3 in fixed shares (launch_xengine_tma_range). The
+// sums are exact (integer values below 2^53 for INT8; the FP64 add of the FP32 sums for FP16),
+// as the dump kernel's.
 template <typename AccT>
 struct SideDump {
     static constexpr int U = 8;             // visibilities per lane and chunk, loads before stores
@@ -324,9 +325,17 @@ struct SideDump {
         c = __shfl_sync(0xffffffffu, c, 0);
         if (c >= n) return false;
         if (lane == 0) prefetch(c + kAhead * gridDim.x);
+        take(c, lane);
+        return true;
+    }
+    // chunk c
+    __device__ __forceinline__ void take(unsigned c, int lane) const {
         const long long e0 = (long long)c * kChunk + lane;
         add(static_cast<const AccT *>(p.side_src) + e0, p.side_dst + e0, p.side_n - e0);
-        return true;
+    }
+    // every share-th chunk from c on
+    __device__ __forceinline__ void fixed(unsigned c, unsigned share, int lane) const {
+        for (; c < n_chunks() && !*abort_flag; c += share) take(c, lane);
     }
 };
 
@@ -915,7 +924,11 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
     if (p.side_n > 0) {
         // deferred dump: warps 2 and 3 from the start, the others when their role has ended
         const SideDump<AccT> side{p, abort_flag};
-        while (side.chunk(lane)) {
+        if (p.side_ctr) {
+            while (side.chunk(lane)) {
+            }
+        } else if (warp == 2 || warp == 3) {
+            side.fixed(2 * blockIdx.x + warp - 2, 2 * gridDim.x, lane);
         }
     }
 
@@ -924,7 +937,7 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
     tc::tc_fence_after();
     if (warp == 1) tc::tmem_dealloc(tmem, 512);
     // every warp of this CTA has had its last claim refused; after the last CTA's, none is made
-    if (threadIdx.x == 0 && p.side_n > 0 && atomicAdd(p.side_ctr + 1, 1u) == gridDim.x - 1) {
+    if (threadIdx.x == 0 && p.side_n > 0 && p.side_ctr && atomicAdd(p.side_ctr + 1, 1u) == gridDim.x - 1) {
         p.side_ctr[0] = 0;
         p.side_ctr[1] = 0;
     }
@@ -1057,8 +1070,7 @@ corr_status launch_xengine_tma_range(const Handle &h, const void *planes, int np
         // the previous integration's deferred dump rides along (all channels, one launch)
         p.side_dst = h.vis64;
         p.side_src = h.pending_src;
-        p.side_ctr = reinterpret_cast<unsigned *>(h.status) + 1;
-        p.side_n = (long long)h.n_chan * h.n_base;  // (small launches: CTAs without tiles join in)
+        p.side_n = (long long)h.n_chan * h.n_base;
     }
     p.status = h.status;
     p.B = h.n_base;
@@ -1074,7 +1086,15 @@ corr_status launch_xengine_tma_range(const Handle &h, const void *planes, int np
         p.st_kb = h.st_block / 64;
         p.st_nchan = h.n_chan;
     }
-    const unsigned grid = (unsigned)(p.n_items < h.n_sm && p.side_n == 0 ? p.n_items : h.n_sm);
+    unsigned grid = (unsigned)(p.n_items < h.n_sm ? p.n_items : h.n_sm);
+    // A dump of up to four chunks (of some 2 us) for each of the idle warps is done by them
+    // alone: the launch takes 8 us in any case, and CTAs without tiles, the claims and the
+    // count at the end only add to it (with dump, us: INT8 48 inputs x 16 channels x 1001
+    // spectra 24.8 -> 22.8; hi/lo 4 x 16 x 33 21.5 -> 16.6). For more, every SM joins in.
+    if (p.side_n > 8ll * SideDump<int2>::kChunk * grid) {
+        p.side_ctr = reinterpret_cast<unsigned *>(h.status) + 1;
+        grid = (unsigned)h.n_sm;
+    }
     StageScope sc(h, CORR_STAGE_XENGINE, st);
     if (h.precision == CORR_PREC_INT8 && p.st_out) {
         using C = TCfg<2, 64>;
