@@ -252,10 +252,12 @@ corr_status note_capture(Handle &h, cudaStream_t st) {
 // The accumulator counts as zero from here on: the next X-engine call stores. cleared: its
 // memory is zero as well.
 corr_status accum_is_zero(Handle &h, cudaStream_t st, bool cleared = false) {
+    // (stale already: nothing has used the accumulator since the event)
+    const bool since = !h.acc_stale;
     h.acc_zero = true;
     h.acc_spectra = 0;
     h.acc_stale = !cleared && !h.capturing;
-    if (h.acc_stale || h.pending_eager) CORR_CUDA_TRY(cudaEventRecord(h.settled_ev, st));
+    if ((h.acc_stale && since) || h.pending_eager) CORR_CUDA_TRY(cudaEventRecord(h.settled_ev, st));
     return CORR_OK;
 }
 
@@ -387,6 +389,7 @@ static corr_status fx_host_run(corr_t *c, const void *volt_host, const float *ch
     CORR_CUDA_TRY(cudaEventRecord(ev[NB + NC + 2 + par], st));
     const bool fused = (h.flags & CORR_FLAG_FUSED_DUMP) != 0;
     const bool store = h.acc_zero;
+    h.acc_stale = false;
     const int cb = (h.n_chan + nc - 1) / nc;
     for (int k = 0; k < nc; ++k) {
         const int c0 = k * cb, c1 = std::min(h.n_chan, c0 + cb);
