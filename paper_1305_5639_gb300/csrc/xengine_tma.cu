@@ -689,7 +689,10 @@ __global__ void __launch_bounds__((WIDE || (ST && MODE == kInt8)) ? NTHREADS_WID
                         for (int q = 0; q < 4; ++q) o[q] = ok[q] ? __ldcg(dst + off[q]) : make_double2(0.0, 0.0);
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            if (ok[q]) dst[off[q]] = add_exact(o[q], val[q]);  // FP32 sums: conversion in integers
+                            // (conversion in integers; stored as data that is not read again, which
+                            // leaves the operands in L2: 2048 inputs x 256 channels x 2048
+                            // spectra 7.65 -> 7.46 ms)
+                            if (ok[q]) __stcs(dst + off[q], add_exact(o[q], val[q]));
                     } else {
                         float2 *dst = p.rect ? static_cast<float2 *>(p.rect_out) + (long long)chan * p.n_p * p.n_q
                                              : static_cast<float2 *>(itm.acc) + (long long)chan * itm.B;
