@@ -289,8 +289,9 @@ CORR_API corr_status corr_restore_vis(corr_t *h, const double *vis_in, void *str
 
 /* The whole step from host memory: raw voltages in, FP64 visibilities out, with
  * the host<->device copies pipelined against the kernels on two library-owned copy
- * streams (8 input blocks: copy-in overlaps the F-engine; 8 channel blocks:
- * X-engine and dump overlap the copy-out of the previous block).
+ * streams (up to 8 input blocks: copy-in overlaps the F-engine; up to 8 channel
+ * blocks: X-engine and dump overlap the copy-out of the previous block; of 2 MB at
+ * least, so that less than 4 MB in, or out, goes as one block that nothing overlaps).
  *   volt_host  [n_in][n_spectra * n_chan] complex int8, host (page-locked memory
  *              lets the copies run asynchronously)
  *   chan_scale [n_chan] float, device (see corr_fengine)

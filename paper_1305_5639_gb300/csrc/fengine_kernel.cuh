@@ -2,8 +2,9 @@
 // Section 2), 8-bit re-packing of the spectra and corner turn to channel-major
 // order, in one pass.
 //
-// Each N = T1 x T2 point FFT is computed by a group of max(T1, T2) threads in two
-// register passes (four-step / Cooley-Tukey split n = t + T2 m, k = k1 + T1 k2):
+// Each N = T1 x T2 point FFT is computed by a group of T2 threads (twice as many where two
+// of them share a column) in two register passes (four-step / Cooley-Tukey split
+// n = t + T2 m, k = k1 + T1 k2):
 //   pass 1: thread t < T2 holds x[t + T2 m], m < T1, and computes the T1-point DFT
 //           over m; the result is multiplied by W_N^(t k1) (twiddle table copied
 //           to shared memory per CTA)
@@ -13,7 +14,7 @@
 // Square lengths (16, 64, 256, 1024) take one thread per column and per row. For T2 = 2 T1
 // (128, 512, 2048) two threads share each row's T2-point DFT, and for 64 x 64 (4096) each
 // column's and each row's (dft_shared): every thread is busy in both passes and holds at
-// most 32 values, so that 16 warps fit on an SM (but FCfg::ONE).
+// most 32 values, so that 16 warps fit on an SM (the power pass at 4096 excepted: FCfg::ONE).
 // A CTA handles one input and SB consecutive spectra; the outputs are staged in
 // shared memory as [channel][spectrum] so that every (channel, input) row segment
 // of SB spectra is written to global memory contiguously (the corner turn). Raw
@@ -809,8 +810,8 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     const int vec_out = (reinterpret_cast<uintptr_t>(out) % 16 == 0) && (f.n_spectra % 8 == 0);
     // blockIdx.x (the spectra block) varies fastest, so the CTAs resident at one time
     // write neighbouring segments of the same output rows
-    // spectra per CTA: SB, or half or a quarter of it (whole rounds of the G FFTs in flight,
-    // whole 16-byte pieces of a row) while the launch has fewer CTAs than the chip has SMs:
+    // spectra per CTA: SB, or half of it (whole rounds of the G FFTs in flight, whole 16-byte
+    // pieces of a row) while the launch has fewer CTAs than the chip has SMs:
     // few inputs and spectra then take the time of one round instead of SB / G of them (7
     // inputs x 80 spectra at N = 4096, one launch per input: 487 -> 396 us
     // for the host pipeline's call)
@@ -821,8 +822,8 @@ corr_status launch_one_(const FShape &f, const void *volt, const float *scale, v
     // for each SM (a CTA ends with one FP64 atomic per channel, and atomics to one address take
     // 16 ns each: with one CTA per block they were all the time of short transforms); parts
     // of a block, whole rounds of the G FFTs in flight, while there are not two CTAs per SM
-    // (one at N = 4096, whose atomics weigh more: 16 inputs x 60 spectra, shared DFTs, 31.8 -> 27.8 us, but
-    // 36.3 with one CTA per block).
+    // (one at N = 4096, whose atomics weigh more: 16 inputs x 60 spectra, shared DFTs, 31.8 -> 27.8
+    // us, but 36.3 with one CTA per block).
     // 128 inputs, int8, us: N = 16 x 32768 spectra 1213 -> 118, N = 64 x 32768 2094 -> 354, N =
     // 256 x 16384 2095 -> 668, N = 512 x 8192 2018 -> 818, N = 1024 x 4096 1332 -> 728, N =
     // 2048 x 2048 1891 -> 996, N = 4096 x 1024 1319 -> 1002.
